@@ -563,52 +563,142 @@ void encode_ops(Pass* p) {
   std::vector<OpWord>* words = &p->words;
   words->clear();
   p->has_perm = p->has_phase = false;
+  // the ops split into flips and phase ops, each with its level
+  struct Prim {
+    uint64_t c[2], t[2];
+    uint32_t level;
+    bool flip;
+  };
+  std::vector<Prim> prims;
+  prims.reserve(2 * ops.size());
+  uint32_t reads[128] = {}, writes[128] = {};   // per qubit: first level after its last
+                                                // reader, its last flip
+  uint32_t levels = 0;
+  auto put = [&](const uint64_t c[2], uint64_t t0, uint64_t t1, bool flip) {
+    Prim q{{c[0], c[1]}, {t0, t1}, 0u, flip};
+    for (int w = 0; w < 2; ++w) {
+      for (uint64_t m = q.c[w]; m; m &= m - 1)
+        q.level = std::max(q.level, writes[64 * w + __builtin_ctzll(m)]);
+      for (uint64_t m = flip ? q.t[w] : 0ull; m; m &= m - 1)
+        q.level = std::max(q.level, reads[64 * w + __builtin_ctzll(m)]);
+    }
+    const uint32_t after = q.level + 1;
+    for (int w = 0; w < 2; ++w) {
+      for (uint64_t m = q.c[w]; m; m &= m - 1) {
+        uint32_t& r = reads[64 * w + __builtin_ctzll(m)];
+        r = std::max(r, after);
+      }
+      for (uint64_t m = flip ? q.t[w] : 0ull; m; m &= m - 1) {
+        uint32_t& r = writes[64 * w + __builtin_ctzll(m)];
+        r = std::max(r, after);
+      }
+    }
+    levels = std::max(levels, after);
+    prims.push_back(q);
+  };
+  // fire slots in op order; slot k's factor is the phase its op applies
+  std::vector<double> factor;
   for (const FOp& o : ops) {
     p->has_perm = p->has_perm || (o.kind & FOP_FLIP);
     p->has_phase = p->has_phase || (o.kind & (FOP_CNT | FOP_PH));
-  }
-  // fire slots in op order; slot k's factor is the phase its op applies
-  std::vector<double> factor;
-  auto form = [](const FOp& o) {
-    if (o.kind == FOP_FLIP) return OPS_FLIP64;
-    if (o.kind == (FOP_FLIP | FOP_HI)) return OPS_FLIP128;
-    return OPS_GEN;
-  };
-  size_t i = 0;
-  while (i < ops.size()) {
-    const uint32_t f = form(ops[i]);
-    size_t j = i;
-    while (j < ops.size() && form(ops[j]) == f) ++j;
-    words->push_back(OpWord{f, (uint32_t)(j - i), 0u, 0u});
-    for (size_t k = i; k < j; ++k) {
-      const FOp& o = ops[k];
-      if (f == OPS_FLIP64) {
-        words->push_back(OpWord{(uint32_t)o.c[0], (uint32_t)(o.c[0] >> 32), (uint32_t)o.t[0],
-                                (uint32_t)(o.t[0] >> 32)});
-        continue;
+    uint64_t w0 = (uint64_t)(o.a0 & 7u) << kOpCountShift;
+    uint64_t w1 = (uint64_t)(o.a1 & 7u) << kOpCountShift;
+    if (o.ph != NO_PH) {
+      const PhasePair& pp = p->phases[o.ph];
+      w0 += 1ull << (factor.size() / 2);
+      factor.push_back(pp.re0);
+      factor.push_back(pp.im0);
+      if (o.sbit != NO_SEL) {
+        w1 += 1ull << (factor.size() / 2);
+        factor.push_back(pp.re1);
+        factor.push_back(pp.im1);
       }
-      FOp e = o;
-      if (f == OPS_GEN) {
-        uint32_t f0 = 0xFF, f1 = 0xFF;
-        if (o.ph != NO_PH) {
-          const PhasePair& pp = p->phases[o.ph];
-          f0 = (uint32_t)(factor.size() / 2);
-          factor.push_back(pp.re0);
-          factor.push_back(pp.im0);
-          if (o.sbit != NO_SEL) {
-            f1 = (uint32_t)(factor.size() / 2);
-            factor.push_back(pp.re1);
-            factor.push_back(pp.im1);
-          }
-        }
-        e.ph = (uint16_t)(f0 | (f1 << 8));
-      }
-      OpWord w[3];
-      static_assert(sizeof(w) == sizeof(FOp), "FOp is three words");
-      std::memcpy(w, &e, sizeof(FOp));
-      words->insert(words->end(), w, w + (f == OPS_FLIP128 ? 2 : 3));
     }
-    i = j;
+    if (w0) put(o.c, w0, 0ull, false);
+    if (o.sbit != NO_SEL && w1 != w0) {
+      uint64_t c[2] = {o.c[0], o.c[1]};
+      c[o.sbit >> 6] |= 1ull << (o.sbit & 63u);
+      put(c, w1 - w0, 0ull, false);
+    }
+    if (o.kind & FOP_FLIP) put(o.c, o.t[0], o.t[1], true);
+  }
+  if (!prims.empty()) {
+    // A phase op may wait, past the levels whose flips it does not read, until
+    // the level before the first later flip of a qubit it reads: all that wait
+    // go out together when one has to, so phase runs are few and long.
+    uint32_t next_flip[128];
+    std::fill(next_flip, next_flip + 128, levels);
+    std::vector<uint32_t> due(levels, 0u);   // some phase op cannot wait past this level
+    for (size_t i = prims.size(); i-- > 0;) {
+      const Prim& q = prims[i];
+      uint32_t until = levels;
+      for (int w = 0; w < 2; ++w)
+        for (uint64_t m = q.flip ? q.t[w] : q.c[w]; m; m &= m - 1) {
+          uint32_t& f = next_flip[64 * w + __builtin_ctzll(m)];
+          if (q.flip) f = std::min(f, q.level);
+          else until = std::min(until, f);
+        }
+      if (!q.flip) due[until - 1] = 1;
+    }
+    std::vector<uint32_t> out_at(levels);    // the phase ops of level l go out after level ..
+    for (uint32_t l = levels, x = levels - 1; l-- > 0;) {
+      if (due[l]) x = l;
+      out_at[l] = x;
+    }
+    for (Prim& q : prims)
+      if (!q.flip) q.level = out_at[q.level];
+    // counting sort by level, flips before phase ops, order kept
+    std::vector<uint32_t> count(2 * (size_t)levels, 0u);
+    std::vector<uint8_t> wide(levels, 0);
+    for (const Prim& q : prims) {
+      ++count[2 * q.level + (q.flip ? 0u : 1u)];
+      if (q.c[1] | (q.flip ? q.t[1] : 0ull)) wide[q.level] = 1;
+    }
+    auto pairs = [&](uint32_t h) { return (count[h] + 1u) / 2u; };
+    for (uint32_t l = 0; l < levels;) {   // narrow stretches shorter than this many steps
+      constexpr uint32_t kMinNarrow = 8;
+      uint32_t e = l, steps = 0;
+      for (; e < levels && !wide[e]; ++e) steps += pairs(2 * e) + pairs(2 * e + 1);
+      if (steps < kMinNarrow && (l > 0 || e < levels)) std::fill(&wide[l], &wide[l] + (e - l), 1);
+      l = e + 1;
+    }
+    // runs: the flips of consecutive levels, up to one with phase ops or a
+    // change of width
+    std::vector<uint32_t> runs;
+    uint32_t flips = 0;
+    for (uint32_t l = 0; l < levels; ++l) {
+      flips += pairs(2 * l);
+      if (pairs(2 * l + 1) || l + 1 == levels || wide[l + 1] != wide[l]) {
+        runs.push_back(flips | pairs(2 * l + 1) << 16u | (wide[l] ? kRunWide : 0u));
+        flips = 0;
+      }
+    }
+    const uint32_t nruns = (uint32_t)runs.size();
+    const uint32_t hdr = 1u + (nruns + 1u + 3u) / 4u;   // one run word past the end is read
+    runs.resize(4 * (size_t)(hdr - 1), 0u);
+    std::vector<uint32_t> next(2 * (size_t)levels);       // next word of each level's halves
+    uint32_t at = hdr;
+    for (uint32_t h = 0; h < 2 * levels; ++h) {
+      next[h] = at;
+      at += 2u * pairs(h) * (wide[h >> 1] ? 2u : 1u);
+    }
+    words->assign((size_t)at + 4u, OpWord{0u, 0u, 0u, 0u});
+    (*words)[0] = OpWord{nruns, hdr, 0u, 0u};
+    std::memcpy(words->data() + 1, runs.data(), runs.size() * sizeof(uint32_t));
+    for (const Prim& q : prims) {
+      uint32_t& pos = next[2 * q.level + (q.flip ? 0u : 1u)];
+      OpWord* w = words->data() + pos;
+      const uint32_t c0 = (uint32_t)q.c[0], c1 = (uint32_t)(q.c[0] >> 32);
+      const uint32_t t0 = (uint32_t)q.t[0], t1 = (uint32_t)(q.t[0] >> 32);
+      if (!wide[q.level]) {
+        w[0] = OpWord{c0, c1, t0, t1};
+        pos += 1;
+      } else {
+        w[0] = OpWord{c0, c1, (uint32_t)q.c[1], (uint32_t)(q.c[1] >> 32)};
+        w[1] = OpWord{t0, t1, (uint32_t)q.t[1], (uint32_t)(q.t[1] >> 32)};
+        pos += 2;
+      }
+    }
   }
   // per-8-slot tables by doubling: entry v = entry (v without its top bit)
   // times the factor of that bit

@@ -142,99 +142,134 @@ __device__ __forceinline__ void unknown_label_masks(Ctl* ctl, uint32_t b) {
   set_label_masks(ctl, b, ~0ull, ~0ull, 0ull, 0ull);
 }
 
-// Runs a fused pass's encoded op stream (OPS_* runs of 16-byte words, in
-// shared or global memory; every thread reads the same word, a broadcast) on
-// E labels at once: flips each label in place, adds the pi/4 steps to cnt and
-// sets the fire-slot bit of every arbitrary phase that applies (the product
-// of those phases is taken afterwards, apply_fire). A label is handled as
-// four 32-bit words, so a condition test or a flip is one three-input logic
-// instruction per word.
+// Predicated, never branched: lanes differ in every condition.
+template <bool WIDE>
+__device__ __forceinline__ void flip_if(uint32_t miss, const uint4& t, uint32_t& w0, uint32_t& w1,
+                                        uint32_t& w2, uint32_t& w3) {
+  if (WIDE)
+    asm("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %8, 0;\n\t@p xor.b32 %0, %0, %4;\n\t"
+        "@p xor.b32 %1, %1, %5;\n\t@p xor.b32 %2, %2, %6;\n\t@p xor.b32 %3, %3, %7;\n\t}"
+        : "+r"(w0), "+r"(w1), "+r"(w2), "+r"(w3)
+        : "r"(t.x), "r"(t.y), "r"(t.z), "r"(t.w), "r"(miss));
+  else
+    asm("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %4, 0;\n\t@p xor.b32 %0, %0, %2;\n\t"
+        "@p xor.b32 %1, %1, %3;\n\t}"
+        : "+r"(w0), "+r"(w1)
+        : "r"(t.x), "r"(t.y), "r"(miss));
+}
+
+__device__ __forceinline__ void add_if(uint32_t miss, const uint4& t, uint64_t& ph) {
+  const uint64_t a = ((uint64_t)t.y << 32) | t.x;
+  asm("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %2, 0;\n\t@p add.u64 %0, %0, %1;\n\t}"
+      : "+l"(ph)
+      : "l"(a), "r"(miss));
+}
+
+// One step of the op stream on E labels: the conditions of both ops are
+// evaluated on the labels as they are before the step (the ops of a level do
+// not read what the others flip), then FLIP: the targets of those that hold
+// are flipped, else their words are added to the labels' phase words. A label
+// is handled as 32-bit words, so a test is one three-input logic instruction a
+// word and a flip one predicated one.
+template <bool WIDE, bool FLIP, int E>
+__device__ __forceinline__ void walk_step(const uint4 (&o)[WIDE ? 4 : 2], uint32_t (&w0)[E],
+                                          uint32_t (&w1)[E], uint32_t (&w2)[E],
+                                          uint32_t (&w3)[E], uint64_t (&ph)[E]) {
+  const uint4 ca = o[0], cb = o[WIDE ? 2 : 1];
+  const uint4 ta = WIDE ? o[1] : make_uint4(ca.z, ca.w, 0u, 0u);
+  const uint4 tb = WIDE ? o[WIDE ? 3 : 1] : make_uint4(cb.z, cb.w, 0u, 0u);
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    uint32_t ma = ((w0[e] & ca.x) ^ ca.x) | ((w1[e] & ca.y) ^ ca.y);
+    uint32_t mb = ((w0[e] & cb.x) ^ cb.x) | ((w1[e] & cb.y) ^ cb.y);
+    if (WIDE) {
+      ma |= ((w2[e] & ca.z) ^ ca.z) | ((w3[e] & ca.w) ^ ca.w);
+      mb |= ((w2[e] & cb.z) ^ cb.z) | ((w3[e] & cb.w) ^ cb.w);
+    }
+    if (FLIP) {
+      flip_if<WIDE>(ma, ta, w0[e], w1[e], w2[e], w3[e]);
+      flip_if<WIDE>(mb, tb, w0[e], w1[e], w2[e], w3[e]);
+    } else {
+      add_if(ma, ta, ph[e]);
+      add_if(mb, tb, ph[e]);
+    }
+  }
+}
+
+// The runs of an op stream from run r on as long as they have this width (see
+// OpWord's comment for the layout); q: the first step. The next step's words
+// are loaded before the current one is worked, so a step costs its own latency
+// and not a load's.
+template <bool WIDE, int E>
+__device__ __forceinline__ void walk_runs(const uint32_t* __restrict__ runs, uint32_t nruns,
+                                          uint32_t& r, const uint4* __restrict__& q,
+                                          uint32_t (&w0)[E], uint32_t (&w1)[E],
+                                          uint32_t (&w2)[E], uint32_t (&w3)[E],
+                                          uint64_t (&ph)[E]) {
+  constexpr int S = WIDE ? 4 : 2;   // words a step
+  uint4 cur[S], nxt[S];
+#pragma unroll
+  for (int i = 0; i < S; ++i) cur[i] = q[i];
+  uint32_t run = runs[r];
+  do {
+    const uint32_t nf = run & 0xFFFFu, np = (run >> 16) & 0x7FFFu;
+    run = runs[++r];
+#pragma unroll 2
+    for (uint32_t k = 0; k < nf; ++k) {
+      q += S;
+#pragma unroll
+      for (int i = 0; i < S; ++i) nxt[i] = q[i];
+      walk_step<WIDE, true, E>(cur, w0, w1, w2, w3, ph);
+#pragma unroll
+      for (int i = 0; i < S; ++i) cur[i] = nxt[i];
+    }
+#pragma unroll 1
+    for (uint32_t k = 0; k < np; ++k) {
+      q += S;
+#pragma unroll
+      for (int i = 0; i < S; ++i) nxt[i] = q[i];
+      walk_step<WIDE, false, E>(cur, w0, w1, w2, w3, ph);
+#pragma unroll
+      for (int i = 0; i < S; ++i) cur[i] = nxt[i];
+    }
+  } while (r < nruns && ((run & kRunWide) != 0u) == WIDE);
+}
+
+// Runs a fused pass's encoded op stream (in shared or global memory; every
+// thread reads the same word, a broadcast) on E labels at once: flips each
+// label in place, sets cnt to the pi/4 steps and fire to the fire-slot bits of
+// the arbitrary phases that apply (the product of those phases is taken
+// afterwards, apply_fire).
 template <int KW, int E>
 __device__ __forceinline__ void walk_ops_n(const uint4* __restrict__ sq, uint32_t nwords,
                                            uint64_t (&k0)[E], uint64_t (&k1)[E],
                                            uint32_t (&cnt)[E], uint64_t (&fire)[E]) {
+  if (nwords == 0u) return;
   uint32_t w0[E], w1[E], w2[E], w3[E];
+  uint64_t ph[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     w0[e] = (uint32_t)k0[e];
     w1[e] = (uint32_t)(k0[e] >> 32);
     w2[e] = (uint32_t)k1[e];
     w3[e] = (uint32_t)(k1[e] >> 32);
+    ph[e] = 0ull;
   }
-  uint32_t pos = 0;
-  while (pos < nwords) {
-    const uint4 h = sq[pos++];
-    const uint32_t count = h.y;
-    if (h.x == OPS_FLIP64) {
-      const uint4* q = sq + pos;
-#pragma unroll 8
-      for (uint32_t j = 0; j < count; ++j) {
-        const uint4 o = q[j];
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-          const uint32_t miss = ((w0[e] & o.x) ^ o.x) | ((w1[e] & o.y) ^ o.y);
-          const uint32_t m = miss == 0u ? ~0u : 0u;
-          w0[e] ^= o.z & m;
-          w1[e] ^= o.w & m;
-        }
-      }
-      pos += count;
-    } else if (h.x == OPS_FLIP128) {
-      const uint4* q = sq + pos;
-#pragma unroll 4
-      for (uint32_t j = 0; j < count; ++j) {
-        const uint4 c = q[2 * j], t = q[2 * j + 1];
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-          uint32_t miss = ((w0[e] & c.x) ^ c.x) | ((w1[e] & c.y) ^ c.y);
-          if (KW == 2) miss |= ((w2[e] & c.z) ^ c.z) | ((w3[e] & c.w) ^ c.w);
-          const uint32_t m = miss == 0u ? ~0u : 0u;
-          w0[e] ^= t.x & m;
-          w1[e] ^= t.y & m;
-          if (KW == 2) {
-            w2[e] ^= t.z & m;
-            w3[e] ^= t.w & m;
-          }
-        }
-      }
-      pos += 2 * count;
-    } else {
-      const uint4* q = sq + pos;
-#pragma unroll 2
-      for (uint32_t j = 0; j < count; ++j) {
-        const uint4 c = q[3 * j], t = q[3 * j + 1];
-        const uint2 meta = *reinterpret_cast<const uint2*>(q + 3 * j + 2);
-        const uint32_t kind = meta.x >> 24;   // a0 | a1 << 8 | sbit << 16 | kind << 24
-        const uint32_t b = (meta.x >> 16) & 0xFFu;
-        const uint32_t f0 = meta.y & 0xFFu, f1 = (meta.y >> 8) & 0xFFu;
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-          uint32_t miss = ((w0[e] & c.x) ^ c.x) | ((w1[e] & c.y) ^ c.y);
-          if (KW == 2) miss |= ((w2[e] & c.z) ^ c.z) | ((w3[e] & c.w) ^ c.w);
-          const bool cond = miss == 0u;
-          bool sel = false;
-          if (kind & FOP_SEL) {
-            const uint32_t word = b < 32 ? w0[e] : b < 64 ? w1[e] : b < 96 ? w2[e] : w3[e];
-            sel = (word >> (b & 31u)) & 1u;
-          }
-          cnt[e] += cond ? (sel ? (meta.x >> 8) & 0xFFu : meta.x & 0xFFu) : 0u;
-          if ((kind & FOP_PH) && cond) fire[e] |= 1ull << (sel ? f1 : f0);
-          const uint32_t m = cond ? ~0u : 0u;
-          w0[e] ^= t.x & m;
-          w1[e] ^= t.y & m;
-          if (KW == 2) {
-            w2[e] ^= t.z & m;
-            w3[e] ^= t.w & m;
-          }
-        }
-      }
-      pos += 3 * count;
-    }
+  const uint2 head = *reinterpret_cast<const uint2*>(sq);   // runs, words before the steps
+  const uint32_t* __restrict__ runs = reinterpret_cast<const uint32_t*>(sq + 1);
+  const uint4* __restrict__ q = sq + head.y;
+  for (uint32_t r = 0; r < head.x;) {
+    if (KW == 2 && (runs[r] & kRunWide) != 0u)
+      walk_runs<true, E>(runs, head.x, r, q, w0, w1, w2, w3, ph);
+    else
+      walk_runs<false, E>(runs, head.x, r, q, w0, w1, w2, w3, ph);
   }
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     k0[e] = ((uint64_t)w1[e] << 32) | w0[e];
     k1[e] = ((uint64_t)w3[e] << 32) | w2[e];
+    cnt[e] = (uint32_t)(ph[e] >> kOpCountShift);
+    fire[e] = ph[e] & ((1ull << kOpCountShift) - 1ull);
   }
 }
 
@@ -262,16 +297,28 @@ __device__ __forceinline__ void cmul_rn(double& re, double& im, double tr, doubl
   im = ni;
 }
 
+// Takes the lowest non-zero byte of fire: its table entry, and fire without it.
+__device__ __forceinline__ double2 next_fire(uint64_t& fire, const double2* __restrict__ tab) {
+  const uint32_t c = (uint32_t)(__ffsll((long long)fire) - 1) >> 3;
+  const uint32_t v = (uint32_t)(fire >> (8u * c)) & 0xFFu;
+  fire &= ~(0xFFull << (8u * c));
+  return tab[c * 256u + v];
+}
+
 // Multiplies an amplitude by the phases of the set fire-slot bits, one table
-// entry (the product of up to 8 slots' phases) per non-zero byte.
+// entry (the product of up to 8 slots' phases) per non-zero byte, the next
+// entry loading while the product with the last one runs. (A loop, not eight
+// predicated products: those would all occupy the FP64 pipe.)
 __device__ __forceinline__ void apply_fire(uint64_t fire, const double2* __restrict__ tab,
                                            double& re, double& im) {
-  for (uint32_t c = 0; fire != 0ull; ++c, fire >>= 8) {
-    const uint32_t v = (uint32_t)(fire & 0xFFull);
-    if (v == 0u) continue;
-    const double2 t = tab[c * 256u + v];
+  if (fire == 0ull) return;
+  double2 t = next_fire(fire, tab);
+  while (fire != 0ull) {
+    const double2 u = next_fire(fire, tab);
     cmul_rn(re, im, t.x, t.y);
+    t = u;
   }
+  cmul_rn(re, im, t.x, t.y);
 }
 
 // Multiplies an amplitude by e^{i pi cnt / 4} (cnt mod 8), exactly for the

@@ -1818,6 +1818,8 @@ static void expand_kw(int e_log2, bool walk, int blocks, int threads, size_t sme
                       Ctl* ctl, Bufs bufs, const ExpandArgs& a, unsigned long long* plog) {
   if (!walk) {
     expand_go<KW, 8, false>(blocks, threads, smem, st, ctl, bufs, a, plog);
+  } else if (e_log2 == 0) {
+    expand_go<KW, 1, true>(blocks, threads, smem, st, ctl, bufs, a, plog);
   } else if (e_log2 == 1) {
     expand_go<KW, 2, true>(blocks, threads, smem, st, ctl, bufs, a, plog);
   } else if (e_log2 == 2) {
@@ -1850,14 +1852,15 @@ int launch_expand(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs, const
   const bool walk = e.nwords > 0;
   const uint64_t total = nnz_bound << e.d;
   // Outputs per lane: 8 without a walk (measured faster than 4 on the 16.8 M
-  // output expansion); with one, as many as still leave about four warps per
-  // SM (more labels per lane share more decode, fewer warps hide less latency).
+  // output expansion); with one, as many as still leave 32 warps per SM, the
+  // rule of launch_fused (the 67-qubit adder on 65,536 outputs: 19 us with one
+  // output a lane, 25 with two, 41 with four).
   int e_log2 = 3;
   if (walk) {
     // lc.max_blocks is the SM count times the resident blocks of lc.threads
     const uint64_t sms = (uint64_t)lc.max_blocks * lc.threads / 2048;
-    const uint64_t warps_wanted = 4ull * (sms ? sms : 1);
-    e_log2 = 1;
+    const uint64_t warps_wanted = 32ull * (sms ? sms : 1);
+    e_log2 = 0;
     while (e_log2 < 3 && total / (32ull << (e_log2 + 1)) >= warps_wanted) ++e_log2;
   }
   const uint64_t span = 32ull << e_log2;

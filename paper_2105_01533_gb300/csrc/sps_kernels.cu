@@ -1336,28 +1336,37 @@ int launch_fused(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs, const 
   a.has_perm = p.has_perm;
   a.has_phase = p.has_phase;
   a.mg = mg;
-  // labels per thread: as many as still leave about four warps per SM per
-  // label slot (SPS_OPT_FUSED_LABELS overrides)
+  // labels per thread: as many as still leave 32 warps per SM
+  // (SPS_OPT_FUSED_LABELS overrides). Sharing an op's decode saves a tenth of a
+  // step's instructions; fewer warps cost more: 65,536 128-bit labels take 26 us
+  // a run of 512 ops with one label a thread, 32 with two and 57 with four, and
+  // 134,596 labels with three ops and one phase 7.5, 8.3 and 12 us with one, two
+  // and eight.
   int e = lanes;
   if (e == 0) {
-    const uint64_t warps_wanted = 4ull * (uint64_t)sm_count(lc);
+    const uint64_t warps_wanted = 32ull * (uint64_t)sm_count(lc);
     e = 1;
     while (e < 8 && nnz_bound / (32ull * (uint64_t)(2 * e)) >= warps_wanted) e *= 2;
   }
   const int blocks = grid_for((nnz_bound + e - 1) / e, lc.threads, lc.max_blocks);
-  // at most 4 words per op: <= 32 KB, under the default 48 KB
   const size_t smem = 16 * (size_t)a.nwords;
   cudaStream_t st = (cudaStream_t)lc.stream;
+  // a run of 512 dependent Y gates on 128-bit labels takes 70 KB
+  auto go = [&](auto kern) {
+    if (smem > 48u * 1024u)
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    kern<<<blocks, lc.threads, smem, st>>>(ctl, bufs, a, plog);
+  };
   if (key_words == 1) {
-    if (e == 1) k_fused<1, 1><<<blocks, lc.threads, smem, st>>>(ctl, bufs, a, plog);
-    else if (e == 2) k_fused<1, 2><<<blocks, lc.threads, smem, st>>>(ctl, bufs, a, plog);
-    else if (e == 4) k_fused<1, 4><<<blocks, lc.threads, smem, st>>>(ctl, bufs, a, plog);
-    else k_fused<1, 8><<<blocks, lc.threads, smem, st>>>(ctl, bufs, a, plog);
+    if (e == 1) go(k_fused<1, 1>);
+    else if (e == 2) go(k_fused<1, 2>);
+    else if (e == 4) go(k_fused<1, 4>);
+    else go(k_fused<1, 8>);
   } else {
-    if (e == 1) k_fused<2, 1><<<blocks, lc.threads, smem, st>>>(ctl, bufs, a, plog);
-    else if (e == 2) k_fused<2, 2><<<blocks, lc.threads, smem, st>>>(ctl, bufs, a, plog);
-    else if (e == 4) k_fused<2, 4><<<blocks, lc.threads, smem, st>>>(ctl, bufs, a, plog);
-    else k_fused<2, 8><<<blocks, lc.threads, smem, st>>>(ctl, bufs, a, plog);
+    if (e == 1) go(k_fused<2, 1>);
+    else if (e == 2) go(k_fused<2, 2>);
+    else if (e == 4) go(k_fused<2, 4>);
+    else go(k_fused<2, 8>);
   }
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
