@@ -326,7 +326,10 @@ typedef enum sps_option {
                                   form, which such a phase run then takes).
                                   Where the form does not apply the usual
                                   kernels run, and the next 1, 2, 4 .. 64
-                                  attempts are skipped. 0: never */,
+                                  attempts are skipped (the next 1 after a run
+                                  that found members absent and was taken as
+                                  groups, see SPS_OPT_FALLBACK_CHAIN; none
+                                  after one that kept every label). 0: never */,
   SPS_OPT_BITSLICE_JIT = 19    /* bit-sliced passes compiled for their run at run
                                   time (NVRTC; the op walk as straight-line code
                                   on registers, every row offset a constant; one
@@ -347,7 +350,12 @@ typedef enum sps_option {
                                   cooperative launch that returns at once when
                                   the attempt took the run and otherwise runs
                                   them in order with grid barriers (the same
-                                  state as their separate launches); 0: each
+                                  state as their separate launches); a run of
+                                  three or more gates is first tried as a whole,
+                                  one butterfly per group of labels that the
+                                  active gates' flips connect (up to 64 members,
+                                  absent ones counted, all groups within the
+                                  capacity); 0: each
                                   pass as its own launches */,
   SPS_OPT_READOUT_MIN_PLANES = 22 /* 8 (default): a registered readout
                                   (sps_set_readout) is summed by the compiled

@@ -90,6 +90,7 @@ struct sps_state {
   uint32_t max_log2 = 8;
   uint64_t table_slots = 0;
   unsigned long long* itab = nullptr;  // gather-form index table
+  GrpCtl* grp = nullptr;               // scratch of the fallback launch's group stage
   uint32_t itab_log2 = 8;
   uint32_t epoch = 0;
   MaskRing masks;             // rotation of the device label-mask buffers
@@ -548,6 +549,8 @@ sps_status sps_create(uint32_t nqubits, uint64_t capacity, void* cuda_stream, sp
   s->itab = (unsigned long long*)p;
   if ((st = dev_alloc(s, sizeof(Ctl), &p)) != SPS_OK) return fail(st);
   s->ctl = (Ctl*)p;
+  if ((st = dev_alloc(s, sizeof(GrpCtl), &p)) != SPS_OK) return fail(st);
+  s->grp = (GrpCtl*)p;
   // partials: 2 per block (the measurement's two sums), then the probability
   // result and the measurement's three results
   if ((st = dev_alloc(s, sizeof(double) * (2 * s->prob_blocks + 4), &p)) != SPS_OK) return fail(st);
@@ -851,9 +854,14 @@ static bool launch_fallback_chain(sps_state* s, const LaunchCfg& lc, const Apply
     }
     s->counters.fused_passes++;
   }
+  const sps_status ge = next_epoch(s, lc);   // the group stage's index
+  if (ge != SPS_OK) {
+    *err = ge;
+    return true;
+  }
   ProfScope ps(s, 11, first_serial, nsteps, 3u);
-  const int n = launch_chain(lc, s->kw, s->ctl, s->bufs, s->itab, steps, nsteps, w, s->nnz_bound,
-                             ps.slot);
+  const int n = launch_chain(lc, s->kw, s->ctl, s->bufs, s->itab, s->grp, s->epoch, steps, nsteps,
+                             w, s->nnz_bound, ps.slot);
   ps.done();
   // (0, a run too large for the launch, was ruled out above)
   if (n <= 0) *err = SPS_ERR_CUDA;

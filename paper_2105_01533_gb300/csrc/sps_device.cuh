@@ -47,9 +47,9 @@ struct LabelMasks { uint64_t or0, or1, and0, and1; };
 
 // The masks in buffer b, reduced over its stripes; every lane of the calling
 // warp (which must be converged) gets them.
-__device__ __forceinline__ LabelMasks read_label_masks(const Ctl* ctl, uint32_t b) {
+__device__ __forceinline__ LabelMasks read_label_masks(const unsigned long long (*lm)[4]) {
   static_assert(kMaskStripes == 32, "one stripe per lane");
-  const unsigned long long* p = ctl->lm[b][threadIdx.x & 31u];
+  const unsigned long long* p = lm[threadIdx.x & 31u];
   LabelMasks m{__ldcg(p), __ldcg(p + 1), __ldcg(p + 2), __ldcg(p + 3)};
   for (int d = 16; d > 0; d >>= 1) {
     m.or0 |= __shfl_xor_sync(0xFFFFFFFFu, m.or0, d);
@@ -60,18 +60,22 @@ __device__ __forceinline__ LabelMasks read_label_masks(const Ctl* ctl, uint32_t 
   return m;
 }
 
+__device__ __forceinline__ LabelMasks read_label_masks(const Ctl* ctl, uint32_t b) {
+  return read_label_masks(ctl->lm[b]);
+}
+
 // No entry can have a partner for a gate whose flip bits are constant over
 // the state (the partner would differ in a constant bit).
 __device__ __forceinline__ bool flip_bits_constant(const LabelMasks& m, const uint64_t f[2]) {
   return (((m.or0 ^ m.and0) & f[0]) | ((m.or1 ^ m.and1) & f[1])) == 0ull;
 }
 
-// Block-wide OR/AND of per-thread label words, merged into one stripe of
-// buffer b with atomics whose results are not waited for (one set per block,
+// Block-wide OR/AND of per-thread label words, merged into one stripe (p) of
+// a mask buffer with atomics whose results are not waited for (one set per block,
 // so the stripes see few atomics each). Every thread of the block must call it;
 // threads without labels pass (0, 0, ~0, ~0).
-__device__ __forceinline__ void merge_label_masks(Ctl* ctl, uint32_t b, uint64_t or0, uint64_t or1,
-                                                  uint64_t and0, uint64_t and1) {
+__device__ __forceinline__ void merge_label_masks(unsigned long long* p, uint64_t or0,
+                                                  uint64_t or1, uint64_t and0, uint64_t and1) {
   __shared__ unsigned long long part[4][32];
   for (int d = 16; d > 0; d >>= 1) {
     or0 |= __shfl_xor_sync(0xFFFFFFFFu, or0, d);
@@ -94,13 +98,17 @@ __device__ __forceinline__ void merge_label_masks(Ctl* ctl, uint32_t b, uint64_t
       and0 &= part[2][w];
       and1 &= part[3][w];
     }
-    unsigned long long* p = ctl->lm[b][blockIdx.x % kMaskStripes];
     if (or0) atomicOr(p, or0);
     if (or1) atomicOr(p + 1, or1);
     if (~and0) atomicAnd(p + 2, and0);
     if (~and1) atomicAnd(p + 3, and1);
   }
   __syncthreads();
+}
+
+__device__ __forceinline__ void merge_label_masks(Ctl* ctl, uint32_t b, uint64_t or0, uint64_t or1,
+                                                  uint64_t and0, uint64_t and1) {
+  merge_label_masks(ctl->lm[b][blockIdx.x % kMaskStripes], or0, or1, and0, and1);
 }
 
 // The masks in buffer b for every thread of the block (all must call it): one

@@ -924,6 +924,27 @@ struct AmpGate {
   uint32_t sbit, qbit, givens, real;
 };
 
+__device__ __forceinline__ AmpGate amp_gate(const BranchOp& op) {
+  AmpGate g;
+  g.c[0] = op.c[0];
+  g.c[1] = op.c[1];
+  g.m[0] = op.m[0];
+  g.m[1] = op.m[1];
+  g.mre[0] = op.m_re[0][0];
+  g.mre[1] = op.m_re[0][1];
+  g.mre[2] = op.m_re[1][0];
+  g.mre[3] = op.m_re[1][1];
+  g.mim[0] = op.m_im[0][0];
+  g.mim[1] = op.m_im[0][1];
+  g.mim[2] = op.m_im[1][0];
+  g.mim[3] = op.m_im[1][1];
+  g.sbit = op.sbit;
+  g.qbit = op.qbit;
+  g.givens = op.givens;
+  g.real = op.real_m;
+  return g;
+}
+
 // 32 x 32 bit transpose over a warp: lane r passes row r (bit c = M[r][c])
 // and gets column `lane` back (bit r = M[r][lane]); block swaps of 16, 8, 4,
 // 2 and 1 over shuffles.
@@ -1226,25 +1247,7 @@ __global__ void __launch_bounds__(256, SPS_AMP_MIN_BLOCKS) k_amp_layer(Ctl* ctl,
   const bool go = ctl->amp_go != 0u;
   if (go) {
     for (uint32_t j = threadIdx.x; j < a.d; j += blockDim.x) {
-      const BranchOp& op = a.ops[j];
-      AmpGate g;
-      g.c[0] = op.c[0];
-      g.c[1] = op.c[1];
-      g.m[0] = op.m[0];
-      g.m[1] = op.m[1];
-      g.mre[0] = op.m_re[0][0];
-      g.mre[1] = op.m_re[0][1];
-      g.mre[2] = op.m_re[1][0];
-      g.mre[3] = op.m_re[1][1];
-      g.mim[0] = op.m_im[0][0];
-      g.mim[1] = op.m_im[0][1];
-      g.mim[2] = op.m_im[1][0];
-      g.mim[3] = op.m_im[1][1];
-      g.sbit = op.sbit;
-      g.qbit = op.qbit;
-      g.givens = op.givens;
-      g.real = op.real_m;
-      sg[j] = g;
+      sg[j] = amp_gate(a.ops[j]);
     }
     if (POST == AMP_PARITY)
       for (uint32_t c = threadIdx.x; c < 2 * a.npar; c += blockDim.x) spar[c] = a.par[c];
@@ -1378,6 +1381,384 @@ __global__ void __launch_bounds__(256, SPS_AMP_MIN_BLOCKS) k_amp_layer(Ctl* ctl,
 }
 
 // ---------------------------------------------------------------------------
+// A run of branching passes on disjoint qubits as groups, for states that the
+// run changes (the sector of a number-conserving circuit while it fills): the
+// first stage of the fallback launch. As in the amplitude-only form a label's
+// group is spanned by the flips of the gates it activates, and the whole run
+// is one butterfly over the group; but members may be absent (amplitude zero),
+// values may be pruned on the way (from then on zero, the same thing), and the
+// survivors are compacted into the other buffer:
+//   grp_build  indexes every label;
+//   grp_grow   a group is worked by its member with every selector bit 0; where
+//              that label is absent, a label of the group appends it behind the
+//              state's entries (amplitude zero) and to the index, so exactly one
+//              entry leads each group;
+//   grp_emit   leaders queue by group size and run rounds as k_amp_layer's; an
+//              entry no gate touches is pruned and copied.
+// The result equals the passes' one after the other bit for bit (up to the
+// sign of zeros), with their update count. Where the form does not hold (a
+// label activating more than 6 gates, leaders or all members of all groups not
+// fitting the capacity, a full index) nothing is published and the passes run:
+// in particular every intermediate state of the run fits the capacity if all
+// members do, so a capacity error is the passes' to find.
+// One build, two lookups a label and one store a survivor replace a build, 2^4
+// lookups a label and a store for every four gates: a layer of 32 Givens on the
+// 635,376-label sector took 1,160 us as eight such passes.
+struct GrpArgs {
+  uint32_t on;           // 0: not tried
+  uint32_t d;            // gates of the run
+  uint32_t epoch;        // of the stage's index
+  uint32_t load_pct, max_log2;
+  uint32_t words_act;    // as AmpArgs
+  double eps2, eps;
+  uint64_t capacity;
+};
+
+template <int KW>
+__device__ __forceinline__ void grp_build(Ctl* ctl, GrpCtl* g, const SoA& s, uint64_t n,
+                                          unsigned long long* itab, uint64_t mask,
+                                          unsigned long long ep) {
+  if (blockIdx.x == 0) {
+    if (threadIdx.x == 0) {
+      ctl->index_ok = 0u;   // slots are taken over
+      g->grown = g->closure = g->total = g->updates = g->chunk = 0ull;
+      g->bad = 0u;
+      g->took = 0u;
+    }
+    for (uint32_t t = threadIdx.x; t < (uint32_t)kMaskStripes; t += blockDim.x) {
+      g->lm[t][0] = g->lm[t][1] = 0ull;
+      g->lm[t][2] = g->lm[t][3] = ~0ull;
+    }
+  }
+  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
+       i += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t hv = hash_label<KW>(s.lo[i], KW == 2 ? s.hi[i] : 0ull);
+    const unsigned long long mine = ep | ((hv >> 48) << 32) | i;
+    uint64_t h = hv & mask;
+    bool ok = false;
+    for (uint64_t p = 0; p <= mask; ++p, h = (h + 1) & mask) {
+      const unsigned long long v = __ldcg(itab + h);
+      if ((v & 0xFFFF000000000000ull) == ep) continue;
+      if (atomicCAS(itab + h, v, mine) == v) {
+        ok = true;
+        break;
+      }
+    }
+    if (!ok) atomicOr(&g->bad, 1u);
+  }
+}
+
+// Makes sure that label (lo, hi), absent from the state or not, is indexed:
+// appends it at the next free entry if it is absent. Two warps may append one
+// label at once: the one that finds the other's slot first in its way marks
+// its entry as empty (all ones, never a label). Returns false where no room is
+// left.
+template <int KW>
+__device__ __forceinline__ bool grp_append(GrpCtl* g, const SoA& s, uint64_t n, uint64_t capacity,
+                                           unsigned long long* itab, uint64_t mask,
+                                           unsigned long long ep, uint64_t lo, uint64_t hi) {
+  const uint64_t hv = hash_label<KW>(lo, hi);
+  const unsigned long long fp = (hv >> 48) << 32;
+  uint64_t h = hv & mask;
+  uint64_t mine = ~0ull;
+  for (uint64_t p = 0; p <= mask;) {
+    unsigned long long v = __ldcg(itab + h);
+    if ((v & 0xFFFF000000000000ull) != ep) {   // free: the label is not indexed
+      if (mine == ~0ull) {
+        const uint64_t at = n + atomicAdd(&g->grown, 1ull);
+        if (at >= capacity || at > 0xFFFFFFFFull) return false;
+        mine = at;
+        s.lo[at] = lo;
+        if (KW == 2) s.hi[at] = hi;
+        s.re[at] = 0.0;
+        s.im[at] = 0.0;
+        __threadfence();   // the entry before its slot
+      }
+      const unsigned long long old = atomicCAS(itab + h, v, ep | fp | mine);
+      if (old == v) return true;
+      v = old;   // another label took the slot: look at it
+    }
+    if ((v & 0x0000FFFF00000000ull) == fp) {
+      const uint64_t j = v & 0xFFFFFFFFull;
+      if (j >= n) __threadfence();   // an entry appended by this launch: after its slot
+      if (__ldcg(s.lo + j) == lo && (KW == 1 || __ldcg(s.hi + j) == hi)) {
+        if (mine != ~0ull) {
+          s.lo[mine] = EMPTY;
+          if (KW == 2) s.hi[mine] = EMPTY;
+        }
+        return true;
+      }
+    }
+    h = (h + 1) & mask;
+    ++p;
+  }
+  return false;
+}
+
+// Active gates of each of the warp's 32 labels, and of those the ones whose
+// selector bit is set.
+__device__ __forceinline__ void grp_active(const AmpGate* sg, uint32_t d, const uint32_t* pl,
+                                           unsigned lane, uint32_t& act, uint32_t& sel) {
+  uint32_t A = 0u, S = 0u;
+  if (lane < d) {
+    const AmpGate& g = sg[lane];
+    A = gate_plane(g, pl);
+    S = A & pl[g.sbit];
+  }
+  act = warp_transpose32(A, lane);
+  sel = warp_transpose32(S, lane);
+}
+
+template <int KW>
+__device__ __forceinline__ void grp_grow(GrpCtl* g, const GrpArgs& a, const AmpGate* sg,
+                                         uint32_t* pl, const SoA& s, uint64_t n,
+                                         unsigned long long* itab, uint64_t mask,
+                                         unsigned long long ep) {
+  const unsigned lane = threadIdx.x & 31u;
+  const uint64_t nwarps = (uint64_t)gridDim.x * (blockDim.x >> 5);
+  bool bad = false;
+  for (uint64_t c = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); c * 32 < n;
+       c += nwarps) {
+    const uint64_t i = c * 32 + lane;
+    const bool valid = i < n;
+    uint64_t k0 = valid ? s.lo[i] : 0ull;
+    uint64_t k1 = (KW == 2 && valid) ? s.hi[i] : 0ull;
+    uint32_t act, sel;
+    label_planes<KW>(pl, k0, k1, a.words_act, lane);
+    grp_active(sg, a.d, pl, lane, act, sel);
+    if (!valid) act = sel = 0u;
+    if (__popc(act) > (int)kAmpMaxActive) {
+      bad = true;
+    } else if (sel != 0u) {
+      for (uint32_t m = sel; m; m &= m - 1u) {
+        const AmpGate& gt = sg[__ffs(m) - 1];
+        k0 ^= gt.m[0];
+        k1 ^= gt.m[1];
+      }
+      if (!grp_append<KW>(g, s, n, a.capacity, itab, mask, ep, k0, k1)) bad = true;
+    }
+    if (__any_sync(FULL, bad)) break;
+  }
+  if (__any_sync(FULL, bad) && lane == 0) atomicOr(&g->bad, 1u);
+}
+
+// What a warp's lanes collect over their rounds.
+struct GrpSums {
+  uint64_t mo0 = 0, mo1 = 0, ma0 = ~0ull, ma1 = ~0ull;   // OR / AND of the written labels
+  unsigned long long updates = 0, members = 0;
+};
+
+// Writes the lanes' surviving entries (keep) behind those of other warps.
+template <int KW>
+__device__ __forceinline__ void grp_store(GrpCtl* g, const SoA& out, uint64_t capacity,
+                                          unsigned lane, bool keep, uint64_t l0, uint64_t l1,
+                                          double re, double im, GrpSums& sum) {
+  const unsigned b = __ballot_sync(FULL, keep);
+  if (b == 0u) return;
+  unsigned long long base = 0ull;
+  if (lane == 0) base = atomicAdd(&g->total, (unsigned long long)__popc(b));
+  base = __shfl_sync(FULL, base, 0);
+  if (!keep) return;
+  const uint64_t pos = base + __popc(b & ((1u << lane) - 1u));
+  if (pos < capacity) {
+    out.lo[pos] = l0;
+    if (KW == 2) out.hi[pos] = l1;
+    out.re[pos] = re;
+    out.im[pos] = im;
+  }
+  sum.mo0 |= l0;
+  sum.mo1 |= l1;
+  sum.ma0 &= l0;
+  sum.ma1 &= l1;
+}
+
+// One round of groups of 2^c members, laid over the lanes as in amp_round.
+template <int KW>
+__device__ __forceinline__ void grp_round(GrpCtl* g, const GrpArgs& a, const AmpGate* sg,
+                                          const SoA& s, const SoA& out, uint64_t n,
+                                          const unsigned long long* itab, uint64_t mask,
+                                          unsigned long long ep, uint64_t eps_bits, uint32_t c,
+                                          const uint32_t* qidx, const uint32_t* qact,
+                                          uint32_t head, uint32_t ng, unsigned lane,
+                                          GrpSums& sum) {
+  const uint32_t lg = c < 5u ? c : 5u;
+  const bool two = c > 5u;
+  const uint32_t gi = lane >> lg;
+  const bool have = gi < ng;
+  uint64_t wi = 0ull, w0 = 0ull, w1 = 0ull;
+  uint32_t wact = 0u;
+  if (have) {
+    const uint32_t slot = (head + gi) % kAmpRing;
+    wi = qidx[slot];
+    wact = qact[slot];
+    w0 = s.lo[wi];
+    w1 = KW == 2 ? s.hi[wi] : 0ull;
+  }
+  uint32_t gidx[kAmpMaxActive];
+  {
+    uint32_t rem = wact;
+#pragma unroll
+    for (uint32_t b = 0; b < kAmpMaxActive; ++b) {
+      gidx[b] = rem ? (uint32_t)(__ffs(rem) - 1) : 0u;
+      rem &= rem - 1u;
+    }
+  }
+  const uint32_t u0 = lane & ((1u << lg) - 1u);
+  double vr[2] = {0.0, 0.0}, vi[2] = {0.0, 0.0};
+  uint64_t m0[2] = {0ull, 0ull}, m1[2] = {0ull, 0ull};
+  bool here[2] = {false, false};   // present after the gates so far
+#pragma unroll
+  for (uint32_t r = 0; r < 2; ++r) {
+    if (!have || (r == 1 && !two)) continue;
+    const uint32_t u = u0 + 32u * r;
+    uint64_t l0 = w0, l1 = w1;
+#pragma unroll
+    for (uint32_t b = 0; b < kAmpMaxActive; ++b)
+      if (b < c && ((u >> b) & 1u)) {
+        const AmpGate& gt = sg[gidx[b]];
+        l0 ^= gt.m[0];
+        l1 ^= gt.m[1];
+      }
+    m0[r] = l0;
+    m1[r] = l1;
+    if (u == 0u) {
+      here[r] = wi < n;   // (an appended leader is absent)
+      vr[r] = s.re[wi];
+      vi[r] = s.im[wi];
+    } else {
+      here[r] = find_entry<KW>(itab, mask, ep, s, l0, l1, &vr[r], &vi[r]) != ~0ull;
+    }
+    sum.members += 1ull;
+    sum.updates += here[r] ? 1u : 0u;   // the run's first gate
+    if ((wact & 1u) == 0u && here[r] && !keep_amp(vr[r], vi[r], a.eps2, eps_bits)) {
+      here[r] = false;   // gates before the first active one prune the inputs
+      vr[r] = vi[r] = 0.0;
+    }
+  }
+  uint32_t counted = 1u;   // gates whose nonzeros before them are counted
+#pragma unroll
+  for (uint32_t b = 0; b < kAmpMaxActive; ++b) {
+    if (b >= c) break;
+    const AmpGate& gt = sg[gidx[b]];
+    const uint32_t before = gidx[b] + 1u - counted;   // this gate and the inactive ones before it
+#pragma unroll
+    for (uint32_t r = 0; r < 2; ++r) sum.updates += here[r] ? before : 0u;
+    counted = gidx[b] + 1u;
+    if (b < 5u) {
+      const bool x = (lane >> b) & 1u;
+#pragma unroll
+      for (uint32_t r = 0; r < 2; ++r) {
+        if (r == 1 && !two) continue;
+        const double pr = __shfl_xor_sync(FULL, vr[r], 1u << b);
+        const double pi = __shfl_xor_sync(FULL, vi[r], 1u << b);
+        gate_row<false>(gt, x ? 1 : 0, x ? pr : vr[r], x ? pi : vi[r], x ? vr[r] : pr,
+                        x ? vi[r] : pi, &vr[r], &vi[r]);
+      }
+    } else {
+      double n0r, n0i, n1r, n1i;
+      gate_row<false>(gt, 0, vr[0], vi[0], vr[1], vi[1], &n0r, &n0i);
+      gate_row<false>(gt, 1, vr[0], vi[0], vr[1], vi[1], &n1r, &n1i);
+      vr[0] = n0r;
+      vi[0] = n0i;
+      vr[1] = n1r;
+      vi[1] = n1i;
+    }
+#pragma unroll
+    for (uint32_t r = 0; r < 2; ++r) {
+      here[r] = have && (r == 0 || two) && keep_amp(vr[r], vi[r], a.eps2, eps_bits);
+      if (!here[r]) vr[r] = vi[r] = 0.0;
+    }
+  }
+#pragma unroll
+  for (uint32_t r = 0; r < 2; ++r) {
+    if (r == 1 && !two) continue;
+    sum.updates += here[r] ? a.d - counted : 0u;
+    grp_store<KW>(g, out, a.capacity, lane, here[r], m0[r], m1[r], vr[r], vi[r], sum);
+  }
+}
+
+template <int KW>
+__device__ __forceinline__ void grp_emit(GrpCtl* g, const GrpArgs& a, const AmpGate* sg,
+                                         uint32_t* pl, uint32_t (*sqi)[kAmpRing],
+                                         uint32_t (*sqa)[kAmpRing], const SoA& s, const SoA& out,
+                                         uint64_t n, uint64_t entries,
+                                         const unsigned long long* itab, uint64_t mask,
+                                         unsigned long long ep) {
+  const unsigned lane = threadIdx.x & 31u;
+  const uint64_t eps_bits = eps_pattern(a.eps);
+  GrpSums sum;
+  uint32_t qhead[kAmpMaxActive], qtail[kAmpMaxActive];   // warp-uniform
+#pragma unroll
+  for (uint32_t c = 0; c < kAmpMaxActive; ++c) qhead[c] = qtail[c] = 0u;
+  const uint64_t nchunks = (entries + 31) / 32;
+  unsigned long long ch = 0ull;
+  if (lane == 0) ch = atomicAdd(&g->chunk, 1ull);
+  ch = __shfl_sync(FULL, ch, 0);
+  for (; ch < nchunks;) {
+    unsigned long long next = 0ull;
+    if (lane == 0) next = atomicAdd(&g->chunk, 1ull);
+    const uint64_t i = ch * 32 + lane;
+    const uint64_t k0 = i < entries ? s.lo[i] : EMPTY;
+    const uint64_t k1 = (KW == 2 && i < entries) ? s.hi[i] : EMPTY;
+    const bool valid = !(k0 == EMPTY && (KW == 1 || k1 == EMPTY));
+    uint32_t act, sel;
+    label_planes<KW>(pl, k0, k1, a.words_act, lane);
+    grp_active(sg, a.d, pl, lane, act, sel);
+    if (!valid) act = 0u;
+    const uint32_t na = __popc(act);
+    const bool leader = act != 0u && sel == 0u;
+    {   // entries no gate touches: counted before each gate, pruned by the first
+      double re = 0.0, im = 0.0;
+      bool keep = false;
+      if (valid && act == 0u) {
+        re = s.re[i];
+        im = s.im[i];
+        keep = keep_amp(re, im, a.eps2, eps_bits);
+        sum.members += 1ull;
+        sum.updates += keep ? a.d : 1u;
+      }
+      grp_store<KW>(g, out, a.capacity, lane, keep, k0, KW == 2 ? k1 : 0ull, re, im, sum);
+    }
+#pragma unroll
+    for (uint32_t c = 1; c <= kAmpMaxActive; ++c) {
+      const bool mine = leader && na == c;
+      const uint32_t Mc = __ballot_sync(FULL, mine);
+      if (Mc == 0u) continue;
+      if (mine) {
+        const uint32_t slot = (qtail[c - 1] + __popc(Mc & ((1u << lane) - 1u))) % kAmpRing;
+        sqi[c - 1][slot] = (uint32_t)i;
+        sqa[c - 1][slot] = act;
+      }
+      qtail[c - 1] += __popc(Mc);
+      __syncwarp();
+      const uint32_t per = 32u >> (c < 5u ? c : 5u);
+      while (qtail[c - 1] - qhead[c - 1] >= per) {
+        grp_round<KW>(g, a, sg, s, out, n, itab, mask, ep, eps_bits, c, sqi[c - 1], sqa[c - 1],
+                      qhead[c - 1], per, lane, sum);
+        qhead[c - 1] += per;
+      }
+    }
+    ch = __shfl_sync(FULL, next, 0);
+  }
+#pragma unroll
+  for (uint32_t c = 1; c <= kAmpMaxActive; ++c) {
+    const uint32_t left = qtail[c - 1] - qhead[c - 1];
+    if (left)
+      grp_round<KW>(g, a, sg, s, out, n, itab, mask, ep, eps_bits, c, sqi[c - 1], sqa[c - 1],
+                    qhead[c - 1], left, lane, sum);
+  }
+  merge_label_masks(g->lm[blockIdx.x % kMaskStripes], sum.mo0, sum.mo1, sum.ma0, sum.ma1);
+  for (int dd = 16; dd > 0; dd >>= 1) {
+    sum.updates += __shfl_xor_sync(FULL, sum.updates, dd);
+    sum.members += __shfl_xor_sync(FULL, sum.members, dd);
+  }
+  if (lane == 0 && sum.members) {
+    atomicAdd(&g->updates, sum.updates);
+    atomicAdd(&g->closure, sum.members);
+  }
+}
+
+// ---------------------------------------------------------------------------
 // The passes an amplitude-only attempt stands in for, in one cooperative
 // launch. When the attempt took the run, block 0 carries the label masks
 // through the passes' buffers (what each skipped emit does) and every block
@@ -1405,6 +1786,7 @@ struct ChainStep {
 
 struct ChainArgs {
   uint32_t nsteps;
+  GrpArgs grp;
   ChainStep steps[kChainSteps];
   WalkArgs w;
 };
@@ -1488,9 +1870,91 @@ __device__ __forceinline__ void chain_walk(Ctl* ctl, Bufs bufs, const WalkArgs& 
   }
 }
 
+__device__ __forceinline__ uint32_t step_serial(const ChainStep& st) {
+  return st.kind == PASS_LAYER ? st.l.pass_serial : st.g.pass_serial;
+}
+__device__ __forceinline__ uint64_t step_tag(const ChainStep& st) {
+  return st.kind == PASS_LAYER ? st.l.fail_tag : st.g.fail_tag;
+}
+__device__ __forceinline__ uint32_t step_masks(const ChainStep& st) {
+  return st.kind == PASS_LAYER ? st.l.mg : st.g.mg;
+}
+
+// The steps' gates as groups (GrpArgs); true if that produced the state. Every
+// block calls it; what decides is read after grid barriers, so all agree.
 template <int KW>
+__device__ __forceinline__ bool chain_groups(Ctl* ctl, Bufs bufs, unsigned long long* itab,
+                                             GrpCtl* g, const ChainArgs& a, uint64_t n) {
+  __shared__ AmpGate sg[kMaxAmpGates];
+  __shared__ uint32_t splanes[8][128];
+  __shared__ uint32_t sqi[8][kAmpMaxActive][kAmpRing];
+  __shared__ uint32_t sqa[8][kAmpMaxActive][kAmpRing];
+  if (__syncthreads_or(ctl->status != 0u)) return false;
+  const GrpArgs& ga = a.grp;
+  const unsigned warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) {
+    uint32_t j = 0;
+    for (uint32_t k = 0; k < a.nsteps; ++k) {
+      const ChainStep& st = a.steps[k];
+      if (st.kind == PASS_LAYER)
+        for (uint32_t q = 0; q < st.l.d; ++q) sg[j++] = amp_gate(st.l.ops[q]);
+      else
+        sg[j++] = amp_gate(st.g.op);
+    }
+  }
+  __syncthreads();
+  const unsigned cur = ctl->cur;
+  const SoA s = pick(bufs, cur);
+  const SoA out = pick(bufs, cur ^ 1u);
+  const uint32_t serial = step_serial(a.steps[0]);
+  const uint64_t tag = step_tag(a.steps[0]);
+  const unsigned long long ep = (unsigned long long)ga.epoch << 48;
+  // sized for the state's labels and a leader for each
+  const uint64_t most = 2 * n < ga.capacity ? 2 * n : ga.capacity;
+  const uint64_t mask = itab_mask(most, ga.load_pct, ga.max_log2);
+  grp_build<KW>(ctl, g, s, n, itab, mask, ep);
+  grid_barrier(ctl, serial, tag);
+  grp_grow<KW>(g, ga, sg, splanes[warp], s, n, itab, mask, ep);
+  grid_barrier(ctl, serial, tag);
+  if (__ldcg(&g->bad) != 0u) return false;
+  const uint64_t all = n + __ldcg(&g->grown);
+  const uint64_t entries = all < ga.capacity ? all : ga.capacity;
+  grp_emit<KW>(g, ga, sg, splanes[warp], sqi[warp], sqa[warp], s, out, n, entries, itab, mask, ep);
+  grid_barrier(ctl, serial, tag);
+  if (blockIdx.x == 0 && threadIdx.x < 32) {
+    // every intermediate state fits if every member of every group does
+    const unsigned long long closure = __ldcg(&g->closure), total = __ldcg(&g->total);
+    if (ctl->status == 0u && closure <= ga.capacity) {
+      const ChainStep& sl = a.steps[a.nsteps - 1];
+      const uint32_t mgl = step_masks(sl);
+      const LabelMasks m = read_label_masks(g->lm);
+      warp_set_label_masks(ctl, mg_wr(mgl), m);
+      warp_set_label_masks(ctl, mg_rs(mgl), LabelMasks{0ull, 0ull, ~0ull, ~0ull});
+      if (threadIdx.x == 0) {
+        ctl->nnz = total;
+        ctl->cur = cur ^ 1u;
+        ctl->updates += __ldcg(&g->updates);
+        // A run that only kept labels would have held in the amplitude-only
+        // form: it is tried next. One that found members absent is most likely
+        // followed by another: no attempt there. (After a run that pruned some
+        // the backoff of failed attempts stands.)
+        if (closure > n || total == n) {
+          ctl->amp_streak = 0u;
+          ctl->amp_backoff = closure > n ? 1u : 0u;
+        }
+        g->took = 1u;
+      }
+    }
+  }
+  grid_barrier(ctl, serial, tag);
+  return __ldcg(&g->took) != 0u;
+}
+
+// GRP: with the group stage (its own instance: the stage's registers would
+// leave the passes two blocks an SM instead of three).
+template <int KW, bool GRP>
 __global__ void __launch_bounds__(256) k_chain(Ctl* ctl, Bufs bufs, unsigned long long* itab,
-                                               const __grid_constant__ ChainArgs a,
+                                               GrpCtl* g, const __grid_constant__ ChainArgs a,
                                                unsigned long long* plog) {
   const uint64_t n0 = ctl->nnz;
   if (amp_took(ctl, 1u)) {
@@ -1498,10 +1962,8 @@ __global__ void __launch_bounds__(256) k_chain(Ctl* ctl, Bufs bufs, unsigned lon
     // empties the next: after the chain the masks of its first input are in
     // the last step's input and output buffers, and its third buffer is empty
     if (blockIdx.x == 0 && threadIdx.x < 32 && ctl->status == 0u && a.nsteps > 0) {
-      const ChainStep& s0 = a.steps[0];
-      const ChainStep& sl = a.steps[a.nsteps - 1];
-      const uint32_t mg0 = s0.kind == PASS_LAYER ? s0.l.mg : s0.g.mg;
-      const uint32_t mgl = sl.kind == PASS_LAYER ? sl.l.mg : sl.g.mg;
+      const uint32_t mg0 = step_masks(a.steps[0]);
+      const uint32_t mgl = step_masks(a.steps[a.nsteps - 1]);
       const LabelMasks m = read_label_masks(ctl, mg_rd(mg0));
       warp_set_label_masks(ctl, mg_rd(mgl), m);
       warp_set_label_masks(ctl, mg_wr(mgl), m);
@@ -1518,10 +1980,11 @@ __global__ void __launch_bounds__(256) k_chain(Ctl* ctl, Bufs bufs, unsigned lon
   if (plog && blockIdx.x == 0 && threadIdx.x == 0) plog[0] = n0;
   uint32_t serial = 0;
   uint64_t tag = 0;
-  for (uint32_t k = 0; k < a.nsteps; ++k) {
+  const bool grouped = GRP && chain_groups<KW>(ctl, bufs, itab, g, a, n0);
+  for (uint32_t k = 0; k < a.nsteps && !grouped; ++k) {
     const ChainStep& st = a.steps[k];
-    serial = st.kind == PASS_LAYER ? st.l.pass_serial : st.g.pass_serial;
-    tag = st.kind == PASS_LAYER ? st.l.fail_tag : st.g.fail_tag;
+    serial = step_serial(st);
+    tag = step_tag(st);
     if (st.kind == PASS_LAYER) {
       layer_build<KW>(ctl, bufs, itab, st.l, nullptr);
       grid_barrier(ctl, serial, tag);
@@ -1577,6 +2040,19 @@ static LayerArgs layer_args(const LayerLaunch& l, uint32_t epoch) {
   return a;
 }
 
+// 32-bit label words (bit w: label bits 32 w ..) with a bit of the mask.
+static uint32_t words_of(uint64_t lo, uint64_t hi) {
+  return ((lo & 0xFFFFFFFFull) ? 1u : 0u) | ((lo >> 32) ? 2u : 0u) |
+         ((hi & 0xFFFFFFFFull) ? 4u : 0u) | ((hi >> 32) ? 8u : 0u);
+}
+// The words whose bit-planes decide whether a label activates the gate.
+static uint32_t act_words(const BranchOp& op) {
+  auto bit = [](uint32_t q) {
+    return words_of(q < 64 ? 1ull << q : 0ull, q >= 64 ? 1ull << (q - 64) : 0ull);
+  };
+  return words_of(op.c[0], op.c[1]) | bit(op.sbit) | (op.givens ? bit(op.qbit) : 0u);
+}
+
 static GatherArgs gather_args(const BranchLaunch& b, uint32_t epoch) {
   GatherArgs a;
   std::memset(&a, 0, sizeof(a));
@@ -1615,14 +2091,15 @@ int launch_layer_part(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
 }
 
 // Resident blocks of k_chain per SM at `threads` (0 if the query fails).
-template <int KW>
+template <int KW, bool GRP>
 static int chain_blocks_per_sm(int threads) {
   static int cached[5] = {-1, -1, -1, -1, -1};   // threads 32 << k, k = 0..3
   int k = 0;
   while (k < 4 && (32 << k) < threads) ++k;
   if (cached[k] < 0) {
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_chain<KW>, threads, 0) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_chain<KW, GRP>, threads, 0) !=
+        cudaSuccess) {
       cudaGetLastError();
       nb = 0;
     }
@@ -1632,8 +2109,9 @@ static int chain_blocks_per_sm(int threads) {
 }
 
 int launch_chain(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
-                 unsigned long long* itab, const ChainStepDesc* steps, uint32_t nsteps,
-                 const ChainWalk& w, uint64_t nnz_bound, unsigned long long* plog) {
+                 unsigned long long* itab, GrpCtl* grp, uint32_t grp_epoch,
+                 const ChainStepDesc* steps, uint32_t nsteps, const ChainWalk& w,
+                 uint64_t nnz_bound, unsigned long long* plog) {
   if (nsteps > kChainSteps || w.npar > kMaxAmpParity) return 0;
   thread_local ChainArgs a;   // ~21 KB: kept off the stack
   std::memset(&a, 0, sizeof(a));
@@ -1642,6 +2120,28 @@ int launch_chain(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
     a.steps[k].kind = steps[k].kind;
     if (steps[k].kind == PASS_LAYER) a.steps[k].l = layer_args(steps[k].lay, steps[k].epoch);
     else a.steps[k].g = gather_args(steps[k].br, steps[k].epoch);
+  }
+  if (nsteps && grp && grp_epoch) {
+    GrpArgs& ga = a.grp;
+    const bool lay = steps[0].kind == PASS_LAYER;
+    ga.on = 1u;
+    ga.epoch = grp_epoch;
+    ga.eps = lay ? steps[0].lay.eps : steps[0].br.eps;
+    ga.eps2 = ga.eps * ga.eps;
+    ga.load_pct = lay ? steps[0].lay.load_pct : steps[0].br.load_pct;
+    ga.max_log2 = lay ? steps[0].lay.max_log2 : steps[0].br.max_log2;
+    ga.capacity = lay ? steps[0].lay.capacity : steps[0].br.capacity;
+    for (uint32_t k = 0; k < nsteps; ++k) {
+      const bool l = steps[k].kind == PASS_LAYER;
+      const uint32_t nd = l ? steps[k].lay.d : 1u;
+      for (uint32_t q = 0; q < nd; ++q) ga.words_act |= act_words(l ? steps[k].lay.ops[q] : steps[k].br.op);
+      ga.d += nd;
+    }
+    // one gate: the gather pass indexes only the labels with a partner and
+    // reads half as much (90 us against 160 at 700,000 entries, 38 against 52
+    // at 115,000); two in one layer pass: about equal (94 and 116, 206 and 163);
+    // three: 350 against 206; the eight passes of a layer of 32: 1,160 and 270
+    if (ga.d < 3u || ga.d > kMaxAmpGates) ga.on = 0u;
   }
   a.w.words = reinterpret_cast<const uint4*>(w.words);
   a.w.ftab = reinterpret_cast<const double2*>(w.ftab);
@@ -1652,16 +2152,17 @@ int launch_chain(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
   for (uint32_t c = 0; c < 2 * w.npar; ++c) a.w.par[c] = w.par[c];
   const int threads = lc.threads < 256 ? lc.threads : 256;
   const int sms = lc.max_blocks * lc.threads / 2048;
-  const int per_sm = key_words == 1 ? chain_blocks_per_sm<1>(threads) : chain_blocks_per_sm<2>(threads);
+  const bool gr = a.grp.on != 0u;
+  const int per_sm = key_words == 1
+                         ? (gr ? chain_blocks_per_sm<1, true>(threads) : chain_blocks_per_sm<1, false>(threads))
+                         : (gr ? chain_blocks_per_sm<2, true>(threads) : chain_blocks_per_sm<2, false>(threads));
   if (per_sm <= 0 || sms <= 0) return 0;
   const int blocks = grid_of(nnz_bound, threads, per_sm * sms < 0x7FFF ? per_sm * sms : 0x7FFF);
-  void* args[] = {&ctl, &bufs, &itab, &a, &plog};
-  const cudaError_t e =
-      key_words == 1
-          ? cudaLaunchCooperativeKernel((const void*)k_chain<1>, dim3(blocks), dim3(threads), args, 0,
-                                        (cudaStream_t)lc.stream)
-          : cudaLaunchCooperativeKernel((const void*)k_chain<2>, dim3(blocks), dim3(threads), args, 0,
-                                        (cudaStream_t)lc.stream);
+  void* args[] = {&ctl, &bufs, &itab, &grp, &a, &plog};
+  const void* kern = key_words == 1 ? (gr ? (const void*)k_chain<1, true> : (const void*)k_chain<1, false>)
+                                    : (gr ? (const void*)k_chain<2, true> : (const void*)k_chain<2, false>);
+  const cudaError_t e = cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3(threads), args, 0,
+                                                    (cudaStream_t)lc.stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return -1;
@@ -1732,20 +2233,8 @@ int launch_amp_part(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
   a.has_phase = l.has_phase;
   a.npar = l.npar;
   for (uint32_t c = 0; c < 2 * l.npar; ++c) a.par[c] = l.par[c];
-  // the label words the kernel reads as bit-planes
-  auto words_of = [](uint64_t lo, uint64_t hi) {
-    return ((lo & 0xFFFFFFFFull) ? 1u : 0u) | ((lo >> 32) ? 2u : 0u) |
-           ((hi & 0xFFFFFFFFull) ? 4u : 0u) | ((hi >> 32) ? 8u : 0u);
-  };
-  auto bit_words = [&](uint32_t q) {
-    return words_of(q < 64 ? 1ull << q : 0ull, q >= 64 ? 1ull << (q - 64) : 0ull);
-  };
   a.words_act = 0u;
-  for (uint32_t j = 0; j < l.d; ++j) {
-    const BranchOp& op = l.ops[j];
-    a.words_act |= words_of(op.c[0], op.c[1]) | bit_words(op.sbit);
-    if (op.givens) a.words_act |= bit_words(op.qbit);
-  }
+  for (uint32_t j = 0; j < l.d; ++j) a.words_act |= act_words(l.ops[j]);
   a.words_par = 0u;
   for (uint32_t c = 0; c < l.npar; ++c) a.words_par |= words_of(l.par[2 * c], l.par[2 * c + 1]);
   cudaStream_t st = (cudaStream_t)lc.stream;

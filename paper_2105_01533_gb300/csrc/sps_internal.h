@@ -358,6 +358,19 @@ struct Ctl {
   unsigned long long chunk_next;
 };
 
+// Scratch of the fallback launch's group stage (k_chain), written and read
+// within one launch.
+struct GrpCtl {
+  unsigned long long grown;     // entries appended as leaders (some given up again)
+  unsigned long long closure;   // members of all groups, and entries no gate touches
+  unsigned long long total;     // entries written
+  unsigned long long updates;   // the run's updates
+  unsigned long long chunk;     // next chunk of 32 entries
+  unsigned int bad;             // the form does not hold
+  unsigned int took;            // it produced the state
+  unsigned long long lm[kMaskStripes][4];   // label masks of the entries written
+};
+
 // Mask buffer indices of one label-writing launch, packed rd | wr << 8 | rs << 16.
 struct MaskRing {
   uint32_t gen = 0;
@@ -544,9 +557,12 @@ struct ChainWalk {
   uint32_t npar;
   uint32_t ngates;       // gates of the run; 0: none after the passes
 };
+// grp, grp_epoch: scratch and index epoch of the group stage, which takes the
+// gates of all steps at once where it can (0: not tried).
 int launch_chain(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
-                 unsigned long long* itab, const ChainStepDesc* steps, uint32_t nsteps,
-                 const ChainWalk& w, uint64_t nnz_bound, unsigned long long* plog);
+                 unsigned long long* itab, GrpCtl* grp, uint32_t grp_epoch,
+                 const ChainStepDesc* steps, uint32_t nsteps, const ChainWalk& w,
+                 uint64_t nnz_bound, unsigned long long* plog);
 // Runs the grid barrier of k_chain on a scratch control block (8 blocks, three
 // barriers; block skip_block misses the first); *status receives the block's
 // status word. Returns 0, or -1 on a CUDA error.

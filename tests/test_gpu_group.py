@@ -1,0 +1,131 @@
+"""The group stage of the fallback launch (runs of three or more branching
+gates on disjoint qubits on states that they change): against the passes as
+separate launches, bit for bit with their update count, and the oracle; where
+it hands the run back (groups over 64 members, members over the capacity)
+and where absent members, pruned values, stored zeros, appended leaders and
+partial rounds meet."""
+
+import numpy as np
+import pytest
+
+from oracle import OracleState
+from paper_2105_01533_gb300 import sps
+from paper_2105_01533_gb300 import workloads as W
+
+from helpers import compare_states
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_2105_01533_gb300 import build as B
+    B.build()
+    sps.load_library()
+    yield
+
+
+def random_state(nq, count, seed, zeros=0):
+    rng = np.random.default_rng(seed)
+    lo = set()
+    while len(lo) < count:
+        lo.add(int(rng.integers(0, 1 << min(nq, 14))))
+    lo = np.array(sorted(lo), np.uint64)
+    rng.shuffle(lo)
+    hi = np.zeros_like(lo)
+    if nq > 64:   # the same values on the top qubits
+        hi = (lo & np.uint64(127)) << np.uint64(nq - 64 - 7)
+        lo = lo >> np.uint64(7)
+    re, im = rng.normal(size=count), rng.normal(size=count)
+    re[:zeros] = 0.0
+    im[:zeros] = 0.0
+    return hi, lo, re, im
+
+
+def layer(nq, kind, gates, rng):
+    """`gates` disjoint gates over the qubits random_state populates."""
+    low = 7 if nq > 64 else min(nq, 14)
+    qs = list(range(low)) + (list(range(nq - 7, nq)) if nq > 64 else [])
+    qs = [qs[i] for i in rng.distinct(len(qs), len(qs))]
+    out = []
+    while len(out) < gates:
+        t = rng.angle()
+        if kind == "givens":
+            out.append(W.Givens(qs.pop(), qs.pop(), t))
+        elif kind == "controlled":
+            out.append(W.Givens(qs.pop(), qs.pop(), t) if len(out) % 2 else
+                       W.Rx(qs.pop(), t, qs.pop()))
+        else:
+            out.append([W.H(qs.pop()), W.Rx(qs.pop(), t)][len(out) % 2] if len(qs) > 1 else
+                       W.Ry(qs.pop(), t))
+    return out
+
+
+def both(nq, init, parts, eps, cap, lay=4):
+    got = []
+    for chain in (1, 0):
+        st = sps.SparseState(nq, cap)
+        st.set_option(sps.SPS_OPT_SMALL_RUN_CAP, 0)
+        st.set_option(sps.SPS_OPT_EXPAND, 0)
+        st.set_option(sps.SPS_OPT_LAYER_GATES, lay)
+        st.set_option(sps.SPS_OPT_FALLBACK_CHAIN, chain)
+        st.set_amplitudes(*init)
+        for g in parts:
+            st.apply(W.to_array(g), eps)
+        try:
+            st.sync()
+            err = None
+        except sps.SpsError as e:
+            err = (e.status, e.failed_gate)
+        got.append((err, st.get_amplitudes(), st.updates()))
+        st.close()
+    (e1, a1, u1), (e0, a0, u0) = got
+    assert e1 == e0
+    for x, y in zip(a1, a0):
+        np.testing.assert_array_equal(x, y)
+    assert u1 == u0
+    return e1, a1
+
+
+@pytest.mark.parametrize("kind,gates", [("givens", 3), ("givens", 6), ("controlled", 4), ("all", 3),
+                                        ("all", 5), ("all", 6), ("all", 7)])
+@pytest.mark.parametrize("nq,count", [(14, 1), (14, 31), (14, 700), (63, 2500), (64, 33),
+                                      (100, 900), (127, 65)])
+def test_runs_equal_their_passes(kind, gates, nq, count):
+    rng = W.SplitMix64(31 * nq + count + gates)
+    init = random_state(nq, count, count + gates, zeros=count // 16)
+    parts = [layer(nq, kind, gates, rng) + [W.CZ(0, 2), W.T(1)] for _ in range(3)]
+    for eps in (0.0, 1e-14, 0.2):
+        err, got = both(nq, init, parts, eps, 1 << 17)
+        assert err is None
+        orc = OracleState(nq)
+        orc.set(*init)
+        for g in parts:
+            orc.apply(W.to_array(g), eps=eps)
+        if eps == 1e-14:   # (at 0 and 0.2 rounding decides which values are kept)
+            compare_states(got, orc.get(), eps, atol=1e-12)
+
+
+@pytest.mark.parametrize("cap", [640, 641, 900, 1279, 1280, 5119, 5120, 6000])
+def test_capacity_edges(cap):
+    """640 labels; three H make up to 5,120: passes that overflow, overflow on
+    the way only, or just fit are reported as by the passes one by one."""
+    init = random_state(20, 640, 5)
+    parts = [[W.H(15), W.H(16), W.H(17)], [W.H(15), W.H(16), W.H(17)]]
+    both(20, init, parts, 1e-14, cap, lay=1)
+
+
+def test_sector_fills_as_its_passes_fill_it():
+    g = W.givens_workload(seed=8, nqubits=70, modes=3, layers=7)
+    parts = [g[3 + 70 * k:3 + 70 * (k + 1)] for k in range(7)]
+    one = [np.array([0], np.uint64), np.array([7], np.uint64), np.array([1.0]), np.array([0.0])]
+    err, got = both(70, one, parts, 1e-14, 60000)
+    assert err is None
+    orc = OracleState(70)
+    orc.set(*one)
+    for p in parts:
+        orc.apply(p, eps=1e-14)
+    compare_states(got, orc.get(), 1e-14)
