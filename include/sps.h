@@ -410,7 +410,7 @@ sps_status sps_tune_cache_lookup(const char* path, uint32_t kw, uint32_t log2pea
 
 /* Exercises the grid barrier that the cooperative fallback launch uses
  * between passes: 8 blocks meet at three barriers whose waits give up after
- * `spins` polls (about 256 ns each); block skip_block (>= 8: none) does not
+ * `spins` polls (under a microsecond each); block skip_block (>= 8: none) does not
  * arrive at the first, so the other blocks' waits run out. *result receives
  * the status the launch recorded: SPS_OK when every block arrived,
  * SPS_ERR_TIMEOUT when a wait ran out (the launch still ends; later barriers

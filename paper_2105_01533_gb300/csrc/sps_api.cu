@@ -793,6 +793,12 @@ static bool launch_fallback_chain(sps_state* s, const LaunchCfg& lc, const Apply
   ChainStepDesc steps[kChainSteps];
   uint32_t nsteps = 0;
   const uint32_t first_serial = s->pass_serial + 1;
+  const sps_status ge = next_epoch(s, lc);   // the group stage's index
+  if (ge != SPS_OK) {
+    *err = ge;
+    return true;
+  }
+  const uint32_t grp_epoch = s->epoch;
   for (size_t k = pi; k < amp_end; ++k) {
     const Pass& q = passes[k];
     ChainStepDesc& d = steps[nsteps++];
@@ -854,13 +860,8 @@ static bool launch_fallback_chain(sps_state* s, const LaunchCfg& lc, const Apply
     }
     s->counters.fused_passes++;
   }
-  const sps_status ge = next_epoch(s, lc);   // the group stage's index
-  if (ge != SPS_OK) {
-    *err = ge;
-    return true;
-  }
   ProfScope ps(s, 11, first_serial, nsteps, 3u);
-  const int n = launch_chain(lc, s->kw, s->ctl, s->bufs, s->itab, s->grp, s->epoch, steps, nsteps,
+  const int n = launch_chain(lc, s->kw, s->ctl, s->bufs, s->itab, s->grp, grp_epoch, steps, nsteps,
                              w, s->nnz_bound, ps.slot);
   ps.done();
   // (0, a run too large for the launch, was ruled out above)

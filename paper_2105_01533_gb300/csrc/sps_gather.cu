@@ -1,20 +1,18 @@
 // Gather-form branching pass on the whole GPU (the insert-once rule of Sec. 3.1).
 //
-//   k_gather_build  every input label claims one slot of an open-addressing
-//                   index table: slot = epoch (16 bits) | fingerprint (16 bits,
-//                   the top of the label's hash) | index (32 bits), claimed
-//                   with a 64-bit CAS. Labels are distinct, so no label
+//   k_gather_build  every input label that may be looked up claims one slot of
+//                   an index table (idx_build). Labels are distinct, so no label
 //                   comparison is needed here. A slot whose epoch differs from
 //                   the pass's is free, so the table needs clearing only when
 //                   the 16-bit epoch wraps. The fingerprint lets a lookup skip
 //                   almost every foreign slot without reading its label.
 //   k_gather_emit   every entry: inactive -> itself; active -> look up the
-//                   partner label (flip mask applied); if the partner exists
-//                   and this entry's selector bit is 0, the partner writes the
-//                   pair; else this entry writes both outputs of the 2x2 action
-//                   (each product and sum rounded once). Outputs are pruned and
-//                   compacted (warp ballot, block scan, one atomic per block);
-//                   the last block publishes the count and flips the buffers.
+//                   partner label (flip mask applied) and write the entry's own
+//                   row of the 2x2 action, and the partner's too if there is no
+//                   partner (each product and sum rounded once). Outputs are
+//                   pruned and compacted (ballots, block scan, one atomic per
+//                   block and step); the last block publishes the count and
+//                   flips the buffers.
 //
 // No amplitude atomics: every output is computed once, so the result equals the
 // scatter form bit for bit.
@@ -68,6 +66,177 @@ __device__ __forceinline__ uint64_t itab_mask(uint64_t n, uint32_t load_pct, uin
   return (1ull << table_log2_for((n + 1) / 2, load_pct, max_log2)) - 1;
 }
 
+// ---- the index table ---------------------------------------------------------------
+// 64-bit slots: epoch (16 bits) | fingerprint (16 bits, the top of the label's
+// hash) | entry (32 bits), in buckets of four (one 32-byte sector; the table is
+// 256-byte aligned and holds at least 256 slots). A label's slots are its
+// bucket's, from the slot its hash names on around the bucket, then the next
+// bucket's in the same order; a slot of another epoch is free. So one sector
+// load decides almost every lookup: a bucket with a free slot ends it.
+constexpr unsigned long long kIdxEpoch = 0xFFFF000000000000ull;
+constexpr unsigned long long kIdxPrint = 0x0000FFFF00000000ull;
+
+__device__ __forceinline__ unsigned long long idx_print(uint64_t hv) { return (hv >> 48) << 32; }
+
+struct IdxBucket { unsigned long long v[4]; };
+
+__device__ __forceinline__ IdxBucket idx_load(const unsigned long long* itab, uint64_t b) {
+  IdxBucket k;
+  asm volatile("ld.global.cg.v4.u64 {%0, %1, %2, %3}, [%4];"
+               : "=l"(k.v[0]), "=l"(k.v[1]), "=l"(k.v[2]), "=l"(k.v[3])
+               : "l"(itab + b));
+  return k;
+}
+
+// Bits 0..3: slots of this epoch with the fingerprint; bit 4: some slot is free.
+__device__ __forceinline__ uint32_t idx_match(const IdxBucket& k, unsigned long long ep,
+                                              unsigned long long fp) {
+  uint32_t m = 0u;
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    if ((k.v[t] & kIdxEpoch) != ep) m |= 16u;
+    else if ((k.v[t] & kIdxPrint) == fp) m |= 1u << t;
+  }
+  return m;
+}
+
+__device__ __forceinline__ unsigned long long idx_slot(const IdxBucket& k, uint32_t t) {
+  return t == 0u ? k.v[0] : t == 1u ? k.v[1] : t == 2u ? k.v[2] : k.v[3];
+}
+
+__device__ __forceinline__ uint64_t idx_entry(const IdxBucket& k, uint32_t t) {
+  return idx_slot(k, t) & 0xFFFFFFFFull;
+}
+
+// Indexes every label of the state that want(lo, hi) names, four a thread and
+// step. A claim exchanges its word (epoch | fingerprint | entry) with the slot's;
+// a word of this epoch that comes back is carried on to the next slot (every
+// slot it passes stays taken, so lookups find it). The four labels' loads are
+// in flight together, and so is each round of their claims. What bounds it is
+// the longest of a warp's chains: with a load and a compare-and-swap a claim,
+// one label after the other, 457,728 labels on 2^20 slots took 32 us, with the
+// bucket loaded first and its first free slot swapped 54 (half the claims lost
+// a race), now 18.
+// Returns false in the threads that found the table full.
+template <int KW, typename Want>
+__device__ __forceinline__ bool idx_build(unsigned long long* itab, uint64_t mask,
+                                          unsigned long long ep, const SoA& s, uint64_t n,
+                                          Want want) {
+  constexpr int U = 4;
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t i0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i0 < n; i0 += U * stride) {
+    uint64_t k0[U], k1[U], at[U];
+    unsigned long long carry[U], old[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint64_t i = i0 + u * stride;
+      k0[u] = i < n ? s.lo[i] : 0ull;
+      k1[u] = (KW == 2 && i < n) ? s.hi[i] : 0ull;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint64_t i = i0 + u * stride;
+      carry[u] = 0ull;   // nothing to claim (no epoch is 0)
+      if (i < n && want(k0[u], k1[u])) {
+        const uint64_t hv = hash_label<KW>(k0[u], k1[u]);
+        at[u] = hv & mask;
+        carry[u] = ep | idx_print(hv) | i;
+      }
+    }
+    for (uint64_t seen = 0; (carry[0] | carry[1] | carry[2] | carry[3]) != 0ull; ++seen) {
+      if (seen > mask) return false;
+      const uint32_t t = (uint32_t)seen & 3u;
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (carry[u] != 0ull) old[u] = atomicExch(itab + ((at[u] & ~3ull) | ((at[u] + t) & 3ull)), carry[u]);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (carry[u] == 0ull) continue;
+        carry[u] = (old[u] & kIdxEpoch) == ep ? old[u] : 0ull;
+        if (t == 3u) at[u] = (at[u] + 4) & mask;
+      }
+    }
+  }
+  return true;
+}
+
+// The entry that holds a label, or ~0; AMP: its amplitude too, loaded together
+// with the candidate's label.
+template <int KW, bool AMP>
+__device__ __forceinline__ uint64_t idx_find(const unsigned long long* itab, uint64_t mask,
+                                             unsigned long long ep, const SoA& s, uint64_t lo,
+                                             uint64_t hi, double* re, double* im) {
+  const uint64_t hv = hash_label<KW>(lo, hi);
+  const unsigned long long fp = idx_print(hv);
+  uint64_t b = hv & mask & ~3ull;
+  for (uint64_t seen = 0; seen <= mask; seen += 4, b = (b + 4) & mask) {
+    const IdxBucket k = idx_load(itab, b);
+    const uint32_t m = idx_match(k, ep, fp);
+    for (uint32_t c = m & 15u; c; c &= c - 1u) {
+      const uint64_t j = idx_entry(k, (uint32_t)__ffs(c) - 1u);
+      const uint64_t l0 = s.lo[j];
+      const uint64_t l1 = KW == 2 ? s.hi[j] : 0ull;
+      double r = 0.0, i = 0.0;
+      if (AMP) {
+        r = s.re[j];
+        i = s.im[j];
+      }
+      if (l0 == lo && (KW == 1 || l1 == hi)) {
+        if (AMP) {
+          *re = r;
+          *im = i;
+        }
+        return j;
+      }
+    }
+    if (m & 16u) return ~0ull;
+  }
+  return ~0ull;
+}
+
+// U lookups of one lane at once, bucket loads in flight together, then the
+// candidates' labels and amplitudes; the few that a bucket does not decide (it
+// is full, or its candidate is another label) go through idx_find.
+template <int KW, int U>
+__device__ __forceinline__ void idx_find_n(const unsigned long long* itab, uint64_t mask,
+                                           unsigned long long ep, const SoA& s,
+                                           const bool (&want)[U], const uint64_t (&lo)[U],
+                                           const uint64_t (&hi)[U], bool (&found)[U],
+                                           double (&re)[U], double (&im)[U]) {
+  uint32_t m[U];
+  uint64_t j[U], l0[U], l1[U];
+  IdxBucket k[U];
+  unsigned long long fp[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    found[u] = false;
+    re[u] = im[u] = 0.0;
+    if (!want[u]) continue;
+    const uint64_t hv = hash_label<KW>(lo[u], hi[u]);
+    fp[u] = idx_print(hv);
+    k[u] = idx_load(itab, hv & mask & ~3ull);
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    m[u] = want[u] ? idx_match(k[u], ep, fp[u]) : 16u;
+    if ((m[u] & 15u) == 0u) continue;
+    j[u] = idx_entry(k[u], (uint32_t)__ffs(m[u]) - 1u);
+    l0[u] = s.lo[j[u]];
+    l1[u] = KW == 2 ? s.hi[j[u]] : 0ull;
+    re[u] = s.re[j[u]];
+    im[u] = s.im[j[u]];
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    if (m[u] == 16u) continue;
+    found[u] = (m[u] & 15u) != 0u && l0[u] == lo[u] && (KW == 1 || l1[u] == hi[u]);
+    if (!found[u]) {
+      re[u] = im[u] = 0.0;
+      found[u] = idx_find<KW, true>(itab, mask, ep, s, lo[u], hi[u], &re[u], &im[u]) != ~0ull;
+    }
+  }
+}
+
 template <int KW>
 __device__ __forceinline__ void gather_build(Ctl* ctl, Bufs bufs, unsigned long long* itab,
                                              const GatherArgs& a, unsigned long long* plog) {
@@ -85,58 +254,67 @@ __device__ __forceinline__ void gather_build(Ctl* ctl, Bufs bufs, unsigned long 
   const SoA s = pick(bufs, ctl->cur);
   const unsigned long long ep = (unsigned long long)a.epoch << 48;
   const BranchOp& op = a.op;
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t k0 = s.lo[i];
-    const uint64_t k1 = KW == 2 ? s.hi[i] : 0ull;
-    // The partner of an active label is active too (flipping the target bits
-    // keeps the controls and the Givens condition), so only active labels are
-    // ever looked up: index those alone.
-    bool active = (k0 & op.c[0]) == op.c[0] && (k1 & op.c[1]) == op.c[1];
-    if (op.givens) active = active && (label_bit(k0, k1, op.sbit) != label_bit(k0, k1, op.qbit));
-    if (!active) continue;
-    const uint64_t hv = hash_label<KW>(k0, k1);
-    const unsigned long long mine = ep | ((hv >> 48) << 32) | i;
-    uint64_t h = hv & mask;
-    bool ok = false;
-    for (uint64_t p = 0; p <= mask; ++p, h = (h + 1) & mask) {
-      const unsigned long long v = __ldcg(itab + h);
-      if ((v & 0xFFFF000000000000ull) == ep) continue;   // taken in this pass
-      if (atomicCAS(itab + h, v, mine) == v) {
-        ok = true;
-        break;
-      }
-      // lost the race: the slot now belongs to this pass, go on
+  // The partner of an active label is active too (flipping the target bits
+  // keeps the controls and the Givens condition), so only active labels are
+  // ever looked up: index those alone.
+  const bool ok = idx_build<KW>(itab, mask, ep, s, n, [&](uint64_t k0, uint64_t k1) {
+    const bool on = (k0 & op.c[0]) == op.c[0] && (k1 & op.c[1]) == op.c[1];
+    return on && (!op.givens || label_bit(k0, k1, op.sbit) != label_bit(k0, k1, op.qbit));
+  });
+  if (!ok) fail(ctl, SPS_ERR_TABLE_FULL, a.pass_serial, a.fail_tag);
+}
+
+// Row x of the action on an active entry with selector bit x (its own output):
+// M[x][x] times its amplitude, plus M[x][1-x] times its partner's where there
+// is one; without a partner also the partner label's output, M[1-x][x] times
+// its amplitude. Rounded as pair_action rounds the pair (a sum with an absent
+// partner's zero adds nothing); half the products of one member working the
+// pair, since a warp issues them for all its lanes.
+__device__ __forceinline__ void own_rows(const BranchOp& op, bool x, bool found, uint64_t lo,
+                                         uint64_t hi, double re, double im, double pr, double pi,
+                                         double* o_re, double* o_im, double* q_re, double* q_im) {
+  if (op.pauli) {
+    // the diagonal is cos, the entry taking a(j) to j ^ x is sin times a power of
+    // i (pauli_pair): a signed, perhaps swapped product
+    const double cs = op.m_re[0][0], sn = op.psin;
+    const uint64_t f0 = found ? lo ^ op.m[0] : lo, f1 = found ? hi ^ op.m[1] : hi;
+    const uint32_t e = op.ny + 3u + 2u * (uint32_t)(__popcll(f0 & op.pz[0]) + __popcll(f1 & op.pz[1]));
+    const double sr = found ? pr : re, si = found ? pi : im;
+    double tr = __dmul_rn(sn, (e & 1u) ? si : sr);
+    double ti = __dmul_rn(sn, (e & 1u) ? sr : si);
+    // i^0: (r, i); i^1: (-i, r); i^2: (-r, -i); i^3: (i, -r)
+    if (((e + 1u) & 2u) != 0u) tr = -tr;
+    if ((e & 2u) != 0u) ti = -ti;
+    *o_re = __dmul_rn(cs, re);
+    *o_im = __dmul_rn(cs, im);
+    if (found) {
+      *o_re = __dadd_rn(*o_re, tr);
+      *o_im = __dadd_rn(*o_im, ti);
+    } else {
+      *q_re = tr;
+      *q_im = ti;
     }
-    if (!ok) {
-      fail(ctl, SPS_ERR_TABLE_FULL, a.pass_serial, a.fail_tag);
-      return;
-    }
+    return;
+  }
+  const int xi = x ? 1 : 0;
+  mat_times(op, xi, xi, re, im, o_re, o_im);
+  if (found) {
+    double tr, ti;
+    mat_times(op, xi, 1 - xi, pr, pi, &tr, &ti);
+    *o_re = __dadd_rn(*o_re, tr);
+    *o_im = __dadd_rn(*o_im, ti);
+  } else {
+    mat_times(op, 1 - xi, xi, re, im, q_re, q_im);
   }
 }
 
-template <int KW>
-__device__ __forceinline__ uint64_t find_label(const unsigned long long* itab, uint64_t mask,
-                                               unsigned long long ep, const SoA& s, uint64_t lo,
-                                               uint64_t hi) {
-  const uint64_t hv = hash_label<KW>(lo, hi);
-  const unsigned long long fp = (hv >> 48) << 32;
-  uint64_t h = hv & mask;
-  for (uint64_t p = 0; p <= mask; ++p, h = (h + 1) & mask) {
-    const unsigned long long v = __ldcg(itab + h);
-    if ((v & 0xFFFF000000000000ull) != ep) return ~0ull;
-    if ((v & 0x0000FFFF00000000ull) != fp) continue;
-    const uint64_t j = v & 0xFFFFFFFFull;
-    if (s.lo[j] == lo && (KW == 1 || s.hi[j] == hi)) return j;
-  }
-  return ~0ull;
-}
-
-template <int KW>
+// U entries a thread and step (blockDim apart): their lookups overlap, and a
+// step takes its output places with one atomic for U * blockDim entries.
+template <int KW, int U>
 __device__ __forceinline__ void gather_emit(Ctl* ctl, Bufs bufs, const unsigned long long* itab,
                                             const GatherArgs& a, unsigned long long* plog) {
-  __shared__ unsigned warp_cnt[32];
-  __shared__ unsigned long long block_base;
+  __shared__ unsigned warp_cnt[2][32];
+  __shared__ unsigned long long block_base[2];
   if (__syncthreads_or(ctl->status != 0u)) return;
   const uint64_t n = ctl->nnz;
   if (amp_took(ctl, a.fallback)) {
@@ -155,91 +333,84 @@ __device__ __forceinline__ void gather_emit(Ctl* ctl, Bufs bufs, const unsigned 
   const BranchOp& op = a.op;
   const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   const unsigned nwarps = blockDim.x >> 5;
+  const unsigned below = (1u << lane) - 1u;
+  const uint64_t eps_bits = eps_pattern(a.eps);
   const bool no_partners = flip_bits_constant(read_label_masks_block(ctl, mg_rd(a.mg)), op.m);
   if (blockIdx.x == 0 && threadIdx.x == 0) reset_label_masks(ctl, mg_rs(a.mg));
   uint64_t mo0 = 0, mo1 = 0, ma0 = ~0ull, ma1 = ~0ull;   // OR / AND of the written labels
-  for (uint64_t base = blockIdx.x * (uint64_t)blockDim.x; base < n;
-       base += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t i = base + threadIdx.x;
-    uint64_t l0 = 0, h0 = 0, l1 = 0, h1 = 0;
-    double v0r = 0, v0i = 0, v1r = 0, v1i = 0;
-    bool w0 = false, w1 = false;
-    if (i < n) {
-      const uint64_t k0 = s.lo[i];
-      const uint64_t k1 = KW == 2 ? s.hi[i] : 0ull;
-      const double re = s.re[i], im = s.im[i];
-      bool active = (k0 & op.c[0]) == op.c[0] && (k1 & op.c[1]) == op.c[1];
-      const bool x = label_bit(k0, k1, op.sbit);
-      if (op.givens) active = active && (x != label_bit(k0, k1, op.qbit));
-      if (!active) {
-        l0 = k0; h0 = k1; v0r = re; v0i = im;
-        w0 = keep_amp(re, im, a.eps2, eps_pattern(a.eps));
-      } else {
-        const uint64_t p0 = k0 ^ op.m[0], p1 = k1 ^ op.m[1];
-        const uint64_t j = no_partners ? ~0ull : find_label<KW>(itab, mask, ep, s, p0, p1);
-        if (j == ~0ull || x) {   // else the partner with selector bit 1 writes the pair
-          const double pre = j != ~0ull ? s.re[j] : 0.0;
-          const double pim = j != ~0ull ? s.im[j] : 0.0;
-          const double a0r = x ? pre : re, a0i = x ? pim : im;
-          const double a1r = x ? re : pre, a1i = x ? im : pim;
-          l0 = x ? p0 : k0; h0 = x ? p1 : k1;
-          l1 = x ? k0 : p0; h1 = x ? k1 : p1;
-          if (op.pauli)
-            pair_action(pauli_pair(op, l0, h0, l1, h1), j != ~0ull, x, a0r, a0i, a1r, a1i, &v0r,
-                        &v0i, &v1r, &v1i);
-          else
-            pair_action(op, j != ~0ull, x, a0r, a0i, a1r, a1i, &v0r, &v0i, &v1r, &v1i);
-          w0 = keep_amp(v0r, v0i, a.eps2, eps_pattern(a.eps));
-          w1 = keep_amp(v1r, v1i, a.eps2, eps_pattern(a.eps));
-        }
-      }
+  unsigned side = 0;   // which half of the shared words this step uses
+  for (uint64_t base = (uint64_t)U * blockIdx.x * blockDim.x; base < n;
+       base += (uint64_t)U * gridDim.x * blockDim.x, side ^= 1u) {
+    uint64_t k0[U], k1[U], p0[U], p1[U];
+    double re[U], im[U], pr[U], pi[U];
+    bool act[U], look[U], found[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint64_t i = base + (uint64_t)u * blockDim.x + threadIdx.x;
+      const bool valid = i < n;
+      k0[u] = valid ? s.lo[i] : 0ull;
+      k1[u] = (KW == 2 && valid) ? s.hi[i] : 0ull;
+      re[u] = valid ? s.re[i] : 0.0;   // (a zero is pruned: nothing past the end is written)
+      im[u] = valid ? s.im[i] : 0.0;
+      act[u] = valid && (k0[u] & op.c[0]) == op.c[0] && (k1[u] & op.c[1]) == op.c[1];
+      if (op.givens)
+        act[u] = act[u] && (label_bit(k0[u], k1[u], op.sbit) != label_bit(k0[u], k1[u], op.qbit));
+      p0[u] = k0[u] ^ op.m[0];
+      p1[u] = k1[u] ^ op.m[1];
+      look[u] = act[u] && !no_partners;
     }
-    if (w0) {
-      mo0 |= l0;
-      mo1 |= h0;
-      ma0 &= l0;
-      ma1 &= h0;
+    idx_find_n<KW, U>(itab, mask, ep, s, look, p0, p1, found, pr, pi);
+    double vr[U], vi[U], qr[U], qi[U];
+    unsigned bo[U], bq[U], cnt = 0u;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      vr[u] = re[u];
+      vi[u] = im[u];
+      qr[u] = qi[u] = 0.0;
+      if (act[u])
+        own_rows(op, label_bit(k0[u], k1[u], op.sbit), found[u], k0[u], k1[u], re[u], im[u], pr[u],
+                 pi[u], &vr[u], &vi[u], &qr[u], &qi[u]);
+      bo[u] = __ballot_sync(FULL, keep_amp(vr[u], vi[u], a.eps2, eps_bits));
+      bq[u] = __ballot_sync(FULL, keep_amp(qr[u], qi[u], a.eps2, eps_bits));
+      cnt += __popc(bo[u]) + __popc(bq[u]);
     }
-    if (w1) {
-      mo0 |= l1;
-      mo1 |= h1;
-      ma0 &= l1;
-      ma1 &= h1;
-    }
-    const unsigned b0 = __ballot_sync(FULL, w0), b1 = __ballot_sync(FULL, w1);
-    if (lane == 0) warp_cnt[warp] = __popc(b0) + __popc(b1);
+    if (lane == 0) warp_cnt[side][warp] = cnt;
     __syncthreads();
     if (warp == 0) {
-      const unsigned v = lane < nwarps ? warp_cnt[lane] : 0u;
+      const unsigned v = lane < nwarps ? warp_cnt[side][lane] : 0u;
       unsigned incl = v;
       for (int d = 1; d < 32; d <<= 1) {
         const unsigned t = __shfl_up_sync(FULL, incl, d);
         if (lane >= (unsigned)d) incl += t;
       }
       const unsigned total = __shfl_sync(FULL, incl, 31);
-      if (lane < nwarps) warp_cnt[lane] = incl - v;
+      if (lane < nwarps) warp_cnt[side][lane] = incl - v;
       if (lane == 0)
-        block_base = total ? atomicAdd(&ctl->out_count, (unsigned long long)total) : 0ull;
+        block_base[side] = total ? atomicAdd(&ctl->out_count, (unsigned long long)total) : 0ull;
     }
     __syncthreads();
-    const unsigned below = (1u << lane) - 1u;
-    uint64_t pos = block_base + warp_cnt[warp] + __popc(b0 & below) + __popc(b1 & below);
-    if (w0) {
-      if (pos < a.capacity) {
-        out.lo[pos] = l0;
-        if (KW == 2) out.hi[pos] = h0;
-        out.re[pos] = v0r;
-        out.im[pos] = v0i;
+    uint64_t pos = block_base[side] + warp_cnt[side][warp];
+    auto put = [&](unsigned b, uint64_t l0, uint64_t l1, double r, double i) {
+      if ((b >> lane) & 1u) {
+        const uint64_t at = pos + __popc(b & below);
+        if (at < a.capacity) {
+          out.lo[at] = l0;
+          if (KW == 2) out.hi[at] = l1;
+          out.re[at] = r;
+          out.im[at] = i;
+        }
+        mo0 |= l0;
+        mo1 |= l1;
+        ma0 &= l0;
+        ma1 &= l1;
       }
-      ++pos;
+      pos += __popc(b);
+    };
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      put(bo[u], k0[u], k1[u], vr[u], vi[u]);
+      put(bq[u], p0[u], p1[u], qr[u], qi[u]);
     }
-    if (w1 && pos < a.capacity) {
-      out.lo[pos] = l1;
-      if (KW == 2) out.hi[pos] = h1;
-      out.re[pos] = v1r;
-      out.im[pos] = v1i;
-    }
-    __syncthreads();
   }
   merge_label_masks(ctl, mg_wr(a.mg), mo0, mo1, ma0, ma1);
   if (threadIdx.x == 0) {
@@ -278,66 +449,12 @@ __global__ void __launch_bounds__(256) k_gather_build(Ctl* ctl, Bufs bufs, unsig
   gather_build<KW>(ctl, bufs, itab, a, plog);
 }
 
-// find_label for a lookup that also wants the entry's amplitude: the probe
-// reads the index four slots (one 32-byte sector) at a time from the slot the
-// hash names, and on a fingerprint match loads the candidate's label and
-// amplitude together (the amplitude is kept if the label matches). The slots
-// are scanned in the order the build claimed them, so the result is
-// find_label's. Returns ~0 if the label is not indexed.
-template <int KW>
-__device__ __forceinline__ uint64_t find_entry(const unsigned long long* itab, uint64_t mask,
-                                               unsigned long long ep, const SoA& s, uint64_t lo,
-                                               uint64_t hi, double* re, double* im) {
-  const uint64_t hv = hash_label<KW>(lo, hi);
-  const unsigned long long fp = (hv >> 48) << 32;
-  uint64_t h = hv & mask;
-  uint64_t seen = 0;
-  if (mask < 3) {   // a table of fewer than 4 slots: one at a time
-    for (uint64_t p = 0; p <= mask; ++p, h = (h + 1) & mask) {
-      const unsigned long long v = __ldcg(itab + h);
-      if ((v & 0xFFFF000000000000ull) != ep) return ~0ull;
-      if ((v & 0x0000FFFF00000000ull) != fp) continue;
-      const uint64_t j = v & 0xFFFFFFFFull;
-      if (s.lo[j] == lo && (KW == 1 || s.hi[j] == hi)) {
-        *re = s.re[j];
-        *im = s.im[j];
-        return j;
-      }
-    }
-    return ~0ull;
-  }
-  while (seen <= mask) {
-    const uint64_t b = h & ~3ull;   // the table is 256-byte aligned: a 32-byte sector
-    unsigned long long v4[4];
-    asm("ld.global.cg.v4.u64 {%0, %1, %2, %3}, [%4];"
-        : "=l"(v4[0]), "=l"(v4[1]), "=l"(v4[2]), "=l"(v4[3])
-        : "l"(itab + b));
-    for (uint32_t k = (uint32_t)(h & 3ull); k < 4u; ++k) {
-      const unsigned long long v = v4[k];
-      ++seen;
-      if ((v & 0xFFFF000000000000ull) != ep) return ~0ull;   // a free slot ends the probe
-      if ((v & 0x0000FFFF00000000ull) != fp) continue;
-      const uint64_t j = v & 0xFFFFFFFFull;
-      const uint64_t l0 = s.lo[j];
-      const uint64_t l1 = KW == 2 ? s.hi[j] : 0ull;
-      const double r = s.re[j], i = s.im[j];
-      if (l0 == lo && (KW == 1 || l1 == hi)) {
-        *re = r;
-        *im = i;
-        return j;
-      }
-    }
-    h = (b + 4) & mask;
-  }
-  return ~0ull;
-}
-
-template <int KW>
+template <int KW, int U>
 __global__ void __launch_bounds__(256) k_gather_emit(Ctl* ctl, Bufs bufs,
                                                      const unsigned long long* itab,
                                                      const __grid_constant__ GatherArgs a,
                                                      unsigned long long* plog) {
-  gather_emit<KW>(ctl, bufs, itab, a, plog);
+  gather_emit<KW, U>(ctl, bufs, itab, a, plog);
 }
 
 // ---------------------------------------------------------------------------
@@ -630,28 +747,10 @@ __device__ __forceinline__ void layer_build(Ctl* ctl, Bufs bufs, unsigned long l
   const uint64_t mask = itab_mask(n, a.load_pct, a.max_log2);
   const SoA s = pick(bufs, ctl->cur);
   const unsigned long long ep = (unsigned long long)a.epoch << 48;
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t k0 = s.lo[i];
-    const uint64_t k1 = KW == 2 ? s.hi[i] : 0ull;
-    if ((layer_active<KW>(a, k0, k1) & pairable) == 0u) continue;   // never looked up
-    const uint64_t hv = hash_label<KW>(k0, k1);
-    const unsigned long long mine = ep | ((hv >> 48) << 32) | i;
-    uint64_t h = hv & mask;
-    bool ok = false;
-    for (uint64_t p = 0; p <= mask; ++p, h = (h + 1) & mask) {
-      const unsigned long long v = __ldcg(itab + h);
-      if ((v & 0xFFFF000000000000ull) == ep) continue;
-      if (atomicCAS(itab + h, v, mine) == v) {
-        ok = true;
-        break;
-      }
-    }
-    if (!ok) {
-      fail(ctl, SPS_ERR_TABLE_FULL, a.pass_serial, a.fail_tag);
-      return;
-    }
-  }
+  const bool ok = idx_build<KW>(itab, mask, ep, s, n, [&](uint64_t k0, uint64_t k1) {
+    return (layer_active<KW>(a, k0, k1) & pairable) != 0u;   // else never looked up
+  });
+  if (!ok) fail(ctl, SPS_ERR_TABLE_FULL, a.pass_serial, a.fail_tag);
 }
 
 template <int KW>
@@ -724,7 +823,7 @@ __device__ __forceinline__ void layer_emit(Ctl* ctl, Bufs bufs, const unsigned l
             ++b;
           }
         }
-        const uint64_t jx = find_label<KW>(itab, mask, ep, s, p0, p1);
+        const uint64_t jx = idx_find<KW, false>(itab, mask, ep, s, p0, p1, nullptr, nullptr);
         if (jx == ~0ull) continue;
         const uint32_t u = u_me ^ sm;
         if ((u & lpos) > (u_me & lpos)) {
@@ -1064,27 +1163,8 @@ __global__ void __launch_bounds__(256) k_amp_index(Ctl* ctl, Bufs bufs, unsigned
     const uint64_t mask = itab_mask(n, a.load_pct, a.max_log2);
     const SoA s = pick(bufs, ctl->cur);
     const unsigned long long ep = (unsigned long long)a.epoch << 48;
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
-         i += (uint64_t)gridDim.x * blockDim.x) {
-      const uint64_t k0 = s.lo[i];
-      const uint64_t k1 = KW == 2 ? s.hi[i] : 0ull;
-      const uint64_t hv = hash_label<KW>(k0, k1);
-      const unsigned long long mine = ep | ((hv >> 48) << 32) | i;
-      uint64_t h = hv & mask;
-      bool ok = false;
-      for (uint64_t p = 0; p <= mask; ++p, h = (h + 1) & mask) {
-        const unsigned long long v = __ldcg(itab + h);
-        if ((v & 0xFFFF000000000000ull) == ep) continue;
-        if (atomicCAS(itab + h, v, mine) == v) {
-          ok = true;
-          break;
-        }
-      }
-      if (!ok) {
-        fail(ctl, SPS_ERR_TABLE_FULL, a.pass_serial, a.fail_tag);
-        break;
-      }
-    }
+    if (!idx_build<KW>(itab, mask, ep, s, n, [](uint64_t, uint64_t) { return true; }))
+      fail(ctl, SPS_ERR_TABLE_FULL, a.pass_serial, a.fail_tag);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -1169,7 +1249,7 @@ __device__ __forceinline__ void amp_round(const AmpArgs& a, const AmpGate* sg, c
       vr[r] = s.re[wi];
       vi[r] = s.im[wi];
     } else {
-      jx[r] = find_entry<KW>(itab, mask, ep, s, l0, l1, &vr[r], &vi[r]);
+      jx[r] = idx_find<KW, true>(itab, mask, ep, s, l0, l1, &vr[r], &vi[r]);
     }
     if (jx[r] == ~0ull) {
       ok = false;
@@ -1430,22 +1510,8 @@ __device__ __forceinline__ void grp_build(Ctl* ctl, GrpCtl* g, const SoA& s, uin
       g->lm[t][2] = g->lm[t][3] = ~0ull;
     }
   }
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t hv = hash_label<KW>(s.lo[i], KW == 2 ? s.hi[i] : 0ull);
-    const unsigned long long mine = ep | ((hv >> 48) << 32) | i;
-    uint64_t h = hv & mask;
-    bool ok = false;
-    for (uint64_t p = 0; p <= mask; ++p, h = (h + 1) & mask) {
-      const unsigned long long v = __ldcg(itab + h);
-      if ((v & 0xFFFF000000000000ull) == ep) continue;
-      if (atomicCAS(itab + h, v, mine) == v) {
-        ok = true;
-        break;
-      }
-    }
-    if (!ok) atomicOr(&g->bad, 1u);
-  }
+  if (!idx_build<KW>(itab, mask, ep, s, n, [](uint64_t, uint64_t) { return true; }))
+    atomicOr(&g->bad, 1u);
 }
 
 // Makes sure that label (lo, hi), absent from the state or not, is indexed:
@@ -1458,39 +1524,42 @@ __device__ __forceinline__ bool grp_append(GrpCtl* g, const SoA& s, uint64_t n, 
                                            unsigned long long* itab, uint64_t mask,
                                            unsigned long long ep, uint64_t lo, uint64_t hi) {
   const uint64_t hv = hash_label<KW>(lo, hi);
-  const unsigned long long fp = (hv >> 48) << 32;
-  uint64_t h = hv & mask;
+  const unsigned long long fp = idx_print(hv);
+  uint64_t at = hv & mask;
   uint64_t mine = ~0ull;
-  for (uint64_t p = 0; p <= mask;) {
-    unsigned long long v = __ldcg(itab + h);
-    if ((v & 0xFFFF000000000000ull) != ep) {   // free: the label is not indexed
+  auto same = [&](uint64_t j) {
+    if (j >= n) __threadfence();   // an entry appended by this launch: after its slot
+    if (__ldcg(s.lo + j) != lo || (KW == 2 && __ldcg(s.hi + j) != hi)) return false;
+    if (mine != ~0ull) {   // the entry appended here is given up
+      s.lo[mine] = EMPTY;
+      if (KW == 2) s.hi[mine] = EMPTY;
+    }
+    return true;
+  };
+  for (uint64_t seen = 0; seen <= mask; seen += 4, at = (at + 4) & mask) {
+    const IdxBucket k = idx_load(itab, at & ~3ull);
+    // already indexed? (a claim that idx_build carried on may lie anywhere in its
+    // bucket, so all of it is looked at before a free slot is taken)
+    for (uint32_t c = idx_match(k, ep, fp) & 15u; c; c &= c - 1u)
+      if (same(idx_entry(k, (uint32_t)__ffs(c) - 1u))) return true;
+    for (uint32_t t = 0; t < 4; ++t) {
+      const uint32_t q = (uint32_t)((at + t) & 3ull);
+      const unsigned long long v = idx_slot(k, q);
+      if ((v & kIdxEpoch) == ep) continue;   // taken when loaded
       if (mine == ~0ull) {
-        const uint64_t at = n + atomicAdd(&g->grown, 1ull);
-        if (at >= capacity || at > 0xFFFFFFFFull) return false;
-        mine = at;
-        s.lo[at] = lo;
-        if (KW == 2) s.hi[at] = hi;
-        s.re[at] = 0.0;
-        s.im[at] = 0.0;
+        const uint64_t e = n + atomicAdd(&g->grown, 1ull);
+        if (e >= capacity || e > 0xFFFFFFFFull) return false;
+        mine = e;
+        s.lo[e] = lo;
+        if (KW == 2) s.hi[e] = hi;
+        s.re[e] = 0.0;
+        s.im[e] = 0.0;
         __threadfence();   // the entry before its slot
       }
-      const unsigned long long old = atomicCAS(itab + h, v, ep | fp | mine);
+      const unsigned long long old = atomicCAS(itab + ((at & ~3ull) | q), v, ep | fp | mine);
       if (old == v) return true;
-      v = old;   // another label took the slot: look at it
+      if ((old & kIdxPrint) == fp && same(old & 0xFFFFFFFFull)) return true;   // appended meanwhile
     }
-    if ((v & 0x0000FFFF00000000ull) == fp) {
-      const uint64_t j = v & 0xFFFFFFFFull;
-      if (j >= n) __threadfence();   // an entry appended by this launch: after its slot
-      if (__ldcg(s.lo + j) == lo && (KW == 1 || __ldcg(s.hi + j) == hi)) {
-        if (mine != ~0ull) {
-          s.lo[mine] = EMPTY;
-          if (KW == 2) s.hi[mine] = EMPTY;
-        }
-        return true;
-      }
-    }
-    h = (h + 1) & mask;
-    ++p;
   }
   return false;
 }
@@ -1626,7 +1695,7 @@ __device__ __forceinline__ void grp_round(GrpCtl* g, const GrpArgs& a, const Amp
       vr[r] = s.re[wi];
       vi[r] = s.im[wi];
     } else {
-      here[r] = find_entry<KW>(itab, mask, ep, s, l0, l1, &vr[r], &vi[r]) != ~0ull;
+      here[r] = idx_find<KW, true>(itab, mask, ep, s, l0, l1, &vr[r], &vi[r]) != ~0ull;
     }
     sum.members += 1ull;
     sum.updates += here[r] ? 1u : 0u;   // the run's first gate
@@ -1798,7 +1867,7 @@ static_assert(sizeof(ChainArgs) <= 32000, "kernel parameter space");
 // wait that lasts more than a few seconds marks the barrier broken and records
 // SPS_ERR_TIMEOUT; a broken barrier lets every later wait through at once, so
 // the launch always ends (later steps see the status and do nothing).
-constexpr uint32_t kBarrierSpins = 1u << 24;   // x ~256 ns sleep: ~4 s
+constexpr uint32_t kBarrierSpins = 1u << 24;   // x ~0.25 us (a poll and its sleep): ~4 s
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
   unsigned v;
@@ -1824,7 +1893,7 @@ __device__ __forceinline__ void grid_barrier(Ctl* ctl, uint32_t pass_serial, uin
           fail(ctl, SPS_ERR_TIMEOUT, pass_serial, fail_tag);
           break;
         }
-        __nanosleep(256);
+        __nanosleep(64);
       }
     }
     __threadfence();
@@ -1992,9 +2061,10 @@ __global__ void __launch_bounds__(256) k_chain(Ctl* ctl, Bufs bufs, unsigned lon
     } else {
       gather_build<KW>(ctl, bufs, itab, st.g, nullptr);
       grid_barrier(ctl, serial, tag);
-      gather_emit<KW>(ctl, bufs, itab, st.g, nullptr);
+      gather_emit<KW, 2>(ctl, bufs, itab, st.g, nullptr);
     }
-    grid_barrier(ctl, serial, tag);
+    // (nothing of this launch reads the last pass's state, unless ...)
+    if (k + 1u < a.nsteps || a.w.ngates || plog) grid_barrier(ctl, serial, tag);
   }
   if (a.w.ngates) {
     chain_walk<KW>(ctl, bufs, a.w);
@@ -2285,10 +2355,15 @@ int launch_gather_part(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
     else
       k_gather_build<2><<<blocks, lc.threads, 0, st>>>(ctl, bufs, itab, a, plog);
   } else {
-    if (key_words == 1)
-      k_gather_emit<1><<<blocks, lc.threads, 0, st>>>(ctl, bufs, itab, a, plog);
-    else
-      k_gather_emit<2><<<blocks, lc.threads, 0, st>>>(ctl, bufs, itab, a, plog);
+    const int u = nnz_bound > (uint64_t)lc.max_blocks * (uint64_t)lc.threads ? 2 : 1;
+    const int eb = grid_of((nnz_bound + u - 1) / u, lc.threads, lc.max_blocks);
+    if (key_words == 1) {
+      if (u == 1) k_gather_emit<1, 1><<<eb, lc.threads, 0, st>>>(ctl, bufs, itab, a, plog);
+      else k_gather_emit<1, 2><<<eb, lc.threads, 0, st>>>(ctl, bufs, itab, a, plog);
+    } else {
+      if (u == 1) k_gather_emit<2, 1><<<eb, lc.threads, 0, st>>>(ctl, bufs, itab, a, plog);
+      else k_gather_emit<2, 2><<<eb, lc.threads, 0, st>>>(ctl, bufs, itab, a, plog);
+    }
   }
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }

@@ -1,0 +1,78 @@
+"""The gather-form branching pass (bucketed index, an entry writing its own row
+of the action) against the scatter form, which shares neither its index nor its
+writers, bit for bit: one entry, warps and blocks not filled, two entries a
+thread (700,001), a table at 90% load so that buckets overflow, stored zeros,
+absent partners, controls, real, complex and Pauli matrices, both label widths."""
+
+import numpy as np
+import pytest
+
+from paper_2105_01533_gb300 import sps
+from paper_2105_01533_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+PAULIS = [((0b11, 0), (0, 0)), ((0b11, 0), (0b11, 0)), ((0b101, 0), (0b1100, 0)),
+          ((1, 0), (0b11, 0))]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_2105_01533_gb300 import build as B
+    B.build()
+    sps.load_library()
+    yield
+
+
+def state(nq, count):
+    """Distinct labels, half of them with a neighbour in bit 0, a few zeros."""
+    rng = np.random.default_rng(count)
+    i = np.arange(count, dtype=np.uint64)
+    odd = np.uint64(2654435761)
+    lo = (((i >> np.uint64(1)) * odd) % np.uint64(1 << 20)) << np.uint64(1) | (i & np.uint64(1))
+    lo[::5] ^= np.uint64(1 << 22)
+    hi = np.zeros_like(lo)
+    if nq > 64:
+        hi = lo & np.uint64(63)
+        lo = lo >> np.uint64(3) | (lo & np.uint64(7)) << np.uint64(61)
+    re, im = rng.normal(size=count), rng.normal(size=count)
+    re[::17] = 0.0
+    im[::17] = 0.0
+    return hi, lo, re, im
+
+
+@pytest.mark.parametrize("load", [50, 90])
+@pytest.mark.parametrize("nq,count", [(24, 1), (24, 33), (40, 511), (63, 4097), (70, 2049), (127, 65),
+                                      (30, 700001), (70, 350003)])
+def test_gather_equals_scatter(nq, count, load):
+    init = state(nq, count)
+    t = 7 if nq < 64 else 66
+    gates = [W.H(0), W.Rx(1, 0.7, 2), W.Givens(0, t, 1.1), W.Ry(t, 0.3), W.Rx(0, 2.2)]
+    got = []
+    for form in (1, 2):
+        st = sps.SparseState(nq, 8 * count + 64)
+        for o, v in ((sps.SPS_OPT_SMALL_RUN_CAP, 0), (sps.SPS_OPT_EXPAND, 0), (sps.SPS_OPT_AMP_ONLY, 0),
+                     (sps.SPS_OPT_LAYER_GATES, 1), (sps.SPS_OPT_BRANCH_FORM, form),
+                     (sps.SPS_OPT_LOAD_FACTOR_PCT, load if form == 2 else 50)):
+            st.set_option(o, v)
+        for eps in (0.0, 0.2):
+            st.set_amplitudes(*init)
+            for g in gates[:3]:
+                st.apply(W.to_array([g]), eps)
+            got.append(st.get_amplitudes() + (st.updates(),))
+            st.set_amplitudes(*init)
+            st.apply(W.to_array(gates[3:]), eps)
+            got.append(st.get_amplitudes() + (st.updates(),))
+            for x, z in PAULIS:
+                st.set_amplitudes(*init)
+                st.pauli_exp(x, z, (0, 0), 0.9, eps)
+                st.pauli_exp(x, z, (1 << 5, 0), -1.3, eps)
+                got.append(st.get_amplitudes() + (st.updates(),))
+        st.close()
+    half = len(got) // 2
+    for a, b in zip(got[:half], got[half:]):
+        for x, y in zip(a, b):
+            np.testing.assert_array_equal(x, y)
