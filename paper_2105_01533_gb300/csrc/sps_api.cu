@@ -685,6 +685,7 @@ static sps_status launch_amp_attempt(sps_state* s, const LaunchCfg& lc, const Br
   l.max_log2 = s->itab_log2;
   l.pass_serial = serial;
   l.fail_tag = tag;
+  l.masks_rd = s->masks.reader();
   if (walk && par) {   // the sign-only run after the run, as a parity
     l.fused_gates = walk->ngates;
     l.npar = (uint32_t)(par->size() / 2);
@@ -1515,7 +1516,10 @@ sps_status sps_get_amplitudes(sps_state* s, uint64_t* key_hi, uint64_t* key_lo, 
   *nnz_out = n;
   if (n > cap) return SPS_ERR_CAPACITY;
   if (n == 0) return SPS_OK;
-  const SoA b = s->bufs.b[s->ctl_host->cur];
+  const unsigned cur = s->ctl_host->cur;   // labels and amplitudes (Ctl::cur)
+  SoA b = s->bufs.b[cur & 1u];
+  b.re = s->bufs.b[(cur ^ (cur >> 1)) & 1u].re;
+  b.im = s->bufs.b[(cur ^ (cur >> 1)) & 1u].im;
   bool ok = cudaMemcpyAsync(key_lo, b.lo, n * 8, cudaMemcpyDefault, s->stream) == cudaSuccess &&
             cudaMemcpyAsync(re, b.re, n * 8, cudaMemcpyDefault, s->stream) == cudaSuccess &&
             cudaMemcpyAsync(im, b.im, n * 8, cudaMemcpyDefault, s->stream) == cudaSuccess;

@@ -19,14 +19,18 @@ struct __align__(16) K128a {
   uint64_t lo, hi;
 };
 
-// Buffer selection without indexing the parameter struct dynamically (which
-// would copy it to local memory).
+// The arrays of the state `cur` names (bit 0: label buffer, bit 1: the
+// amplitudes are in the other one), without indexing the parameter struct
+// dynamically (which would copy it to local memory). pick(b, cur ^ 1) are the
+// arrays an out-of-place pass writes; pick(b, cur ^ 2) the same labels with
+// the other amplitudes.
 __device__ __forceinline__ SoA pick(const Bufs& b, unsigned cur) {
+  const bool l = (cur & 1u) != 0u, a = ((cur ^ (cur >> 1)) & 1u) != 0u;
   SoA s;
-  s.lo = cur ? b.b[1].lo : b.b[0].lo;
-  s.hi = cur ? b.b[1].hi : b.b[0].hi;
-  s.re = cur ? b.b[1].re : b.b[0].re;
-  s.im = cur ? b.b[1].im : b.b[0].im;
+  s.lo = l ? b.b[1].lo : b.b[0].lo;
+  s.hi = l ? b.b[1].hi : b.b[0].hi;
+  s.re = a ? b.b[1].re : b.b[0].re;
+  s.im = a ? b.b[1].im : b.b[0].im;
   return s;
 }
 

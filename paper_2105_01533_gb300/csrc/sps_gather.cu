@@ -160,12 +160,19 @@ __device__ __forceinline__ bool idx_build(unsigned long long* itab, uint64_t mas
   return true;
 }
 
+// The high word of an entry's label; s.hi null: every label's is hic.
+template <int KW>
+__device__ __forceinline__ uint64_t high_word(const SoA& s, uint64_t j, uint64_t hic) {
+  return KW == 2 ? (s.hi ? s.hi[j] : hic) : 0ull;
+}
+
 // The entry that holds a label, or ~0; AMP: its amplitude too, loaded together
 // with the candidate's label.
 template <int KW, bool AMP>
 __device__ __forceinline__ uint64_t idx_find(const unsigned long long* itab, uint64_t mask,
                                              unsigned long long ep, const SoA& s, uint64_t lo,
-                                             uint64_t hi, double* re, double* im) {
+                                             uint64_t hi, double* re, double* im,
+                                             uint64_t hic = 0ull) {
   const uint64_t hv = hash_label<KW>(lo, hi);
   const unsigned long long fp = idx_print(hv);
   uint64_t b = hv & mask & ~3ull;
@@ -175,7 +182,7 @@ __device__ __forceinline__ uint64_t idx_find(const unsigned long long* itab, uin
     for (uint32_t c = m & 15u; c; c &= c - 1u) {
       const uint64_t j = idx_entry(k, (uint32_t)__ffs(c) - 1u);
       const uint64_t l0 = s.lo[j];
-      const uint64_t l1 = KW == 2 ? s.hi[j] : 0ull;
+      const uint64_t l1 = high_word<KW>(s, j, hic);
       double r = 0.0, i = 0.0;
       if (AMP) {
         r = s.re[j];
@@ -974,8 +981,8 @@ __global__ void __launch_bounds__(256) k_layer_emit(Ctl* ctl, Bufs bufs,
 // disjoint qubits). Where every active label finds each member of its group
 // and no value on the way falls below eps or to zero, the run maps the set of
 // labels onto itself: the state after it has the same labels, in the same
-// places, with new amplitudes, and each entry is written to the same index of
-// the other buffer (no compaction). A label's group is spanned by the flips of
+// places, with new amplitudes: only those are written, to the same places of
+// the other amplitude arrays (so a failed attempt leaves the state as it was). A label's group is spanned by the flips of
 // the gates it activates; its member with every selector bit 0 (the writer)
 // takes the group: one lane looks up the partner of a pair; a group of 4, 8 or
 // 16 members takes 16 lanes, one per member, that look up their members in
@@ -988,6 +995,13 @@ __global__ void __launch_bounds__(256) k_layer_emit(Ctl* ctl, Bufs bufs,
 // pruned, a group of more than 64) leaves the run to the usual kernels launched after it (fallback = 1), and a
 // failed attempt makes the following runs skip the attempt for a while (1, 2,
 // 4 ... up to 64 runs), so states that keep changing do not pay for it.
+// What bounds a large state (75 M entries, 10.0 ms a layer of 32 Givens) is
+// random sectors, 40 G loads and 28 G stores a second from regions of 2 GB,
+// beside the FP64 products (6 ms): a member costs its index bucket, its label,
+// its two amplitude words and their two stores. Writing the labels beside the
+// amplitudes, and reading a high word that all labels share, cost two stores
+// and a read more: 13.0 ms. (Amplitudes as pairs, one sector where two arrays are
+// two, halved the sectors and took 9.8 ms, less than their conversion costs.)
 struct AmpArgs {
   BranchOp ops[kMaxAmpGates];
   uint32_t d;
@@ -1006,6 +1020,7 @@ struct AmpArgs {
   // 32-bit label words (bit w: label bits 32 w ..) the gates' conditions and
   // selectors read, and those the sign conditions read
   uint32_t words_act, words_par;
+  uint32_t masks_rd;   // label-mask buffer of the state
 };
 
 constexpr int AMP_PLAIN = 0, AMP_WALK = 1, AMP_PARITY = 2;
@@ -1140,8 +1155,6 @@ __device__ __forceinline__ void amp_store(const AmpArgs& a, const uint4* fsm, co
       apply_pi4(cnt, re, im);
     }
   }
-  out.lo[j] = k0;
-  if (KW == 2) out.hi[j] = k1;
   out.re[j] = re;
   out.im[j] = im;
 }
@@ -1203,7 +1216,7 @@ __device__ __forceinline__ void amp_round(const AmpArgs& a, const AmpGate* sg, c
                                           uint64_t mask, unsigned long long ep, uint64_t eps_bits,
                                           uint32_t c, const uint32_t* qidx, const uint32_t* qact,
                                           uint32_t head, uint32_t ng, unsigned lane, bool& bad,
-                                          unsigned long long& written) {
+                                          unsigned long long& written, uint64_t hic) {
   const uint32_t lg = c < 5u ? c : 5u;   // a group takes 2^lg lanes
   const bool two = c > 5u;               // 64 members: u and u + 32 on one lane
   const uint32_t gi = lane >> lg;
@@ -1215,7 +1228,7 @@ __device__ __forceinline__ void amp_round(const AmpArgs& a, const AmpGate* sg, c
     wi = qidx[slot];
     wact = qact[slot];
     w0 = s.lo[wi];
-    w1 = KW == 2 ? s.hi[wi] : 0ull;
+    w1 = high_word<KW>(s, wi, hic);
   }
   uint32_t gidx[kAmpMaxActive];   // the group's gates, in run order
   {
@@ -1249,7 +1262,7 @@ __device__ __forceinline__ void amp_round(const AmpArgs& a, const AmpGate* sg, c
       vr[r] = s.re[wi];
       vi[r] = s.im[wi];
     } else {
-      jx[r] = idx_find<KW, true>(itab, mask, ep, s, l0, l1, &vr[r], &vi[r]);
+      jx[r] = idx_find<KW, true>(itab, mask, ep, s, l0, l1, &vr[r], &vi[r], hic);
     }
     if (jx[r] == ~0ull) {
       ok = false;
@@ -1325,6 +1338,8 @@ __global__ void __launch_bounds__(256, SPS_AMP_MIN_BLOCKS) k_amp_layer(Ctl* ctl,
   __shared__ uint32_t sqa[8][kAmpMaxActive][kAmpRing];   // and their active gates
   extern __shared__ uint4 fsm[];                   // AMP_WALK: the phase run's op stream
   const bool go = ctl->amp_go != 0u;
+  LabelMasks lm{};
+  if (KW == 2 && go) lm = read_label_masks(ctl, a.masks_rd);
   if (go) {
     for (uint32_t j = threadIdx.x; j < a.d; j += blockDim.x) {
       sg[j] = amp_gate(a.ops[j]);
@@ -1343,8 +1358,13 @@ __global__ void __launch_bounds__(256, SPS_AMP_MIN_BLOCKS) k_amp_layer(Ctl* ctl,
   if (go) {
     const uint64_t mask = itab_mask(ctl->index_n, a.load_pct, a.max_log2);
     const unsigned long long ep = (unsigned long long)ctl->index_epoch << 48;
-    const SoA s = pick(bufs, cur);
-    const SoA out = pick(bufs, cur ^ 1u);
+    SoA s = pick(bufs, cur);
+    const SoA out = pick(bufs, cur ^ 2u);   // the labels stay where they are
+    uint64_t hic = 0ull;
+    if (KW == 2 && lm.or1 == lm.and1) {   // one high word for all labels: not read
+      s.hi = nullptr;
+      hic = lm.or1;
+    }
     const uint64_t eps_bits = eps_pattern(a.eps);
     uint32_t* pl = splanes[warp];
     const uint32_t scan_words = a.words_act | (POST == AMP_PARITY ? a.words_par : 0u);
@@ -1363,7 +1383,7 @@ __global__ void __launch_bounds__(256, SPS_AMP_MIN_BLOCKS) k_amp_layer(Ctl* ctl,
       const uint64_t i = ch * 32 + lane;
       const bool valid = i < n;
       const uint64_t k0 = valid ? s.lo[i] : 0ull;
-      const uint64_t k1 = (KW == 2 && valid) ? s.hi[i] : 0ull;
+      const uint64_t k1 = (KW == 2 && valid) ? high_word<KW>(s, i, hic) : 0ull;
       // 1. active gates and writers
       label_planes<KW>(pl, k0, k1, scan_words, lane);
       uint32_t A = 0u, S = 0u;
@@ -1406,7 +1426,7 @@ __global__ void __launch_bounds__(256, SPS_AMP_MIN_BLOCKS) k_amp_layer(Ctl* ctl,
         while (qtail[c - 1] - qhead[c - 1] >= per) {
           amp_round<KW, REAL, POST>(a, sg, spar, pl, fsm, s, out, itab, mask, ep, eps_bits, c,
                                     sqi[warp][c - 1], sqa[warp][c - 1], qhead[c - 1], per, lane,
-                                    bad, written);
+                                    bad, written, hic);
           qhead[c - 1] += per;
         }
       }
@@ -1421,7 +1441,7 @@ __global__ void __launch_bounds__(256, SPS_AMP_MIN_BLOCKS) k_amp_layer(Ctl* ctl,
         if (left)
           amp_round<KW, REAL, POST>(a, sg, spar, pl, fsm, s, out, itab, mask, ep, eps_bits, c,
                                     sqi[warp][c - 1], sqa[warp][c - 1], qhead[c - 1], left, lane,
-                                    bad, written);
+                                    bad, written, hic);
       }
     }
     // every entry written exactly once, or some group had no writer
@@ -1438,7 +1458,7 @@ __global__ void __launch_bounds__(256, SPS_AMP_MIN_BLOCKS) k_amp_layer(Ctl* ctl,
       const bool took = go && atomicAdd(&ctl->amp_fail, 0u) == 0u &&
                         atomicAdd(&ctl->out_count, 0ull) == n;
       if (took) {
-        ctl->cur = cur ^ 1u;
+        ctl->cur = cur ^ 2u;   // the other amplitudes, the same labels
         // no entry appears or goes between the gates (nor in the phase run)
         ctl->updates += n * (a.d + (POST != AMP_PLAIN ? a.fused_gates : 0u));
         ctl->amp_state = 1u;
@@ -2303,6 +2323,7 @@ int launch_amp_part(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
   a.has_phase = l.has_phase;
   a.npar = l.npar;
   for (uint32_t c = 0; c < 2 * l.npar; ++c) a.par[c] = l.par[c];
+  a.masks_rd = l.masks_rd;
   a.words_act = 0u;
   for (uint32_t j = 0; j < l.d; ++j) a.words_act |= act_words(l.ops[j]);
   a.words_par = 0u;

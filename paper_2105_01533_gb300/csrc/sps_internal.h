@@ -325,7 +325,9 @@ constexpr int kMaskStripes = 32;
 struct Ctl {
   unsigned long long nnz;        // entries in the current buffer
   unsigned long long out_count;  // compaction output counter of the running pass
-  unsigned int cur;              // which of the two buffers holds the state
+  unsigned int cur;              // bit 0: the buffer that holds the labels; bit 1: the
+                                 // amplitudes are in the other one (an amplitude-only
+                                 // run flips it, other writers flip bit 0)
   unsigned int status;           // first device-side error (sps_status), 0 = none
   unsigned int fail_pass;        // pass serial of the failing pass
   unsigned int blocks_done;      // last-block detection in the compaction
@@ -531,6 +533,7 @@ struct AmpLaunch {
   // odd number of the npar conditions (c0, c1 pairs: all bits set) hold
   uint64_t par[2 * kMaxAmpParity];
   uint32_t npar;
+  uint32_t masks_rd;   // label-mask buffer of the state
 };
 int launch_amp_part(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
                     unsigned long long* itab, uint32_t epoch, uint32_t force, const AmpLaunch& l,

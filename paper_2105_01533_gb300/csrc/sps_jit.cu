@@ -228,7 +228,10 @@ extern "C" __global__ void __launch_bounds__(128, LB_MIN) k_bs_jit(const JArgs a
   const Soa s = a.b[1];
 #else
   const u32 cur = *reinterpret_cast<volatile u32*>(ctl + OFF_CUR);
-  const Soa s = cur ? a.b[1] : a.b[0];
+  // bit 0: label buffer; bit 1: the amplitudes are in the other one
+  Soa s = (cur & 1u) ? a.b[1] : a.b[0];
+  s.re = ((cur ^ (cur >> 1)) & 1u) ? a.b[1].re : a.b[0].re;
+  s.im = ((cur ^ (cur >> 1)) & 1u) ? a.b[1].im : a.b[0].im;
 #endif
   const unsigned lane = threadIdx.x & 31u;
   const unsigned warp = threadIdx.x >> 5;

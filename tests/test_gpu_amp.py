@@ -326,3 +326,65 @@ def test_grid_barrier_wait_is_bounded():
     st.apply(W.to_array([W.H(q) for q in range(6)]), 0.0)
     assert st.nnz() == 64
     st.close()
+
+
+@pytest.mark.parametrize("n", [24, 70])
+def test_readers_and_writers_after_runs_that_keep_labels(n):
+    """An amplitude-only run writes only amplitudes, to the other buffer's arrays,
+    so labels and amplitudes may lie in different buffers: every other reader
+    and writer after an odd or even number of such runs (readout, phase and
+    permutation passes, an expansion, an out-of-place pass, a failed attempt, a
+    one-block run, a Pauli exponential, read-back, measurement, a reset) sees the
+    state that the runs without the form leave, bit for bit up to the
+    measurement (which scales by sums over another entry order)."""
+    d, top = 12, n - 1
+    spread = [W.H(q) for q in range(d)] + [W.Rz(q, 0.1 + 0.05 * q) for q in range(d)]
+    layer = [W.Ry(q, 0.3 + 0.1 * q) for q in range(5)]
+
+    def after(st, k):
+        if k == 0:
+            return [st.probability((5, 0), (1, 0))]
+        if k == 1:
+            st.apply(W.to_array([W.CX(2, 7), W.T(3), W.P(4, 0.4, 1)]), 1e-14)
+        elif k == 2:
+            st.apply(W.to_array([W.H(top)]), 1e-14)
+        elif k == 3:
+            st.apply(W.to_array([W.X(1), W.H(9), W.H(10, top), W.Rx(11, 0.2)]), 1e-14)
+        elif k == 4:
+            st.pauli_exp((0b11, 0), (0b110, 0), (0, 0), 0.3, 1e-14)
+        elif k == 5:
+            st.apply(W.to_array([W.H(3), W.Z(3), W.H(3)]), 1e-14)
+        return []
+
+    def go(amp):
+        st = sps.SparseState(n, 1 << 14)
+        st.set_option(sps.SPS_OPT_AMP_ONLY, amp)
+        st.apply(W.to_array(spread), 1e-14)
+        seen, whole = [], []
+        for k in range(6):
+            for _ in range(1 + k % 3):
+                st.apply(W.to_array(layer), 1e-14)
+            seen += after(st, k)
+            st.apply(W.to_array(layer[1:]), 1e-14)
+            whole.append(st.get_amplitudes())
+        upd = st.updates()
+        st.apply(W.to_array(layer), 1e-14)
+        seen += st.measure(top, 0.4) + st.measure(0, 0.7)
+        seen += st.measure(1, 0.2) + st.measure(2, 0.6)
+        st.apply(W.to_array(layer), 1e-14)      # (small enough for one block)
+        last = st.get_amplitudes()
+        st.apply(W.to_array(layer), 1e-14)
+        st.reset()
+        st.apply(W.to_array([W.X(2), W.H(1)]), 1e-14)
+        small = st.get_amplitudes()
+        st.close()
+        return seen, whole, upd, last, small
+
+    seen, whole, upd, last, small = go(1)
+    seen0, whole0, upd0, last0, small0 = go(0)
+    for a, b in zip(whole, whole0):
+        identical(a, b)
+    identical(small, small0)
+    assert upd == upd0
+    compare_states(last, last0, 1e-14)
+    np.testing.assert_allclose(seen, seen0, rtol=0, atol=1e-12)
