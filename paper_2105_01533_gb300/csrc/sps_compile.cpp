@@ -792,11 +792,14 @@ bool build_bitslice_expand(const Pass& ex, const Pass& run, uint32_t nqubits, do
   comb.phases.insert(comb.phases.end(), run.phases.begin(), run.phases.end());
   if (comb.phases.size() > kMaxFusedPhases + kMaxExpandGates) return false;
   build_bitslice_rows(comb, nqubits, targets, true, out);
-  if (out->aux_bits > kBsDirectBits) return false;   // the phase from one table
+  // products of chunk entries keep 2^-61 of the common factor's modulus: enough
+  // where every slot's factor has modulus one, not for rotations in the head
+  if (!out->direct && out->aux_bits > 0 && base > 0) return false;
   out->expand = true;
   out->ex_d = ex.ex_d;
   out->c_re = cr;
   out->c_im = ci;
+  std::frexp(std::hypot(cr, ci), &out->c_exp);
   out->row_choice.assign(out->nrows, (int8_t)-1);
   for (uint32_t j = 0; j < ex.ex_d; ++j) {
     const int q = choice_qubit[j];

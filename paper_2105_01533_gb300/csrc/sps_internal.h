@@ -114,7 +114,9 @@ constexpr uint32_t kBsMaxChunkBits = 18; // aux bits per phase table (4 MiB)
 constexpr uint64_t kBsJitMinNnz = 1ull << 20;   // SPS_OPT_BITSLICE_JIT = 1: from this bound
 // Runs with at most this many aux bits get one table of every aux pattern's
 // phase as doubles (2^bits x 16 B, 64 MiB at most): a lookup per entry and no
-// product; more aux bits use fixed-point chunk tables and products.
+// product; more aux bits use fixed-point chunk tables and products (in the
+// expansion form the first chunk's table holds the common factor too, scaled
+// by a power of two, so an output is a fixed-point product and two conversions).
 constexpr uint32_t kBsDirectBits = 22;
 
 struct BsPass {
@@ -155,10 +157,12 @@ struct BsPass {
   // the launch generates the expansion's outputs instead of reading a state.
   // row_choice[r] = the choice bit (output index bit) that label row r holds,
   // -1 for a row of zeros; every label word is written; c_re, c_im = the
-  // factor common to every output; ex_d = the expansion's gates.
+  // factor common to every output, of modulus in [2^(c_exp - 1), 2^c_exp); ex_d =
+  // the expansion's gates.
   bool expand = false;
   std::vector<int8_t> row_choice;
   double c_re = 1.0, c_im = 0.0;
+  int c_exp = 1;
   uint32_t ex_d = 0;
   // aux_bits <= kBsDirectBits: the kernels look the phase up in one table of
   // 2^aux_bits doubles (re, im) built from the (two) fixed-point chunk tables

@@ -22,6 +22,7 @@
 //                    block to finish adds them in block order).
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 
@@ -511,11 +512,11 @@ __device__ __forceinline__ long long q62_mul(long long a, long long b) {
 }
 
 __global__ void k_bs_tables(const longlong2* factors, longlong2* out, uint32_t bits,
-                            uint32_t shift) {
+                            uint32_t shift, longlong2 first) {
   const uint32_t size = 1u << bits;
   for (uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x; idx < size;
        idx += gridDim.x * blockDim.x) {
-    long long re = 1ll << 62, im = 0;
+    long long re = first.x, im = first.y;
     for (uint32_t m = idx; m; m &= m - 1u) {
       const longlong2 f = factors[shift + __ffs(m) - 1u];
       const long long r = q62_mul(re, f.x) - q62_mul(im, f.y);
@@ -1379,9 +1380,15 @@ int launch_bs_tables(const LaunchCfg& lc, const BsLaunch& b) {
   for (uint32_t c = 0; c < P.nchunks; ++c) {
     const uint32_t size = 1u << P.chunk_bits[c];
     const int blocks = (int)((size + 255) / 256);
+    // entry 0: one, or the common factor of an expansion whose outputs are
+    // products of chunk entries
+    longlong2 first = make_longlong2(1ll << 62, 0ll);
+    if (c == 0 && P.expand && !P.direct)
+      first = make_longlong2(std::llround(std::ldexp(P.c_re, 62 - P.c_exp)),
+                             std::llround(std::ldexp(P.c_im, 62 - P.c_exp)));
     k_bs_tables<<<blocks, 256, 0, (cudaStream_t)lc.stream>>>(
         reinterpret_cast<const longlong2*>(b.factors), reinterpret_cast<longlong2*>(b.tables) + toff,
-        P.chunk_bits[c], P.chunk_shift[c]);
+        P.chunk_bits[c], P.chunk_shift[c], first);
     toff += size;
     ++launched;
   }

@@ -135,3 +135,34 @@ def test_adder67_w24_after_reset_closed_form():
     np.testing.assert_array_equal(lo, keys[order])
     err = max(float(np.max(np.abs(re - cre[order]))), float(np.max(np.abs(im - cim[order]))))
     assert err <= 1e-12, err
+
+
+@pytest.mark.parametrize("n,d,cps", [(30, 5, 26), (40, 11, 34), (67, 12, 40), (70, 13, 55)])
+def test_more_phase_bits_than_one_table(n, d, cps):
+    """More than 22 aux bits: an output's phase and the common factor as a product
+    of chunk tables' entries in the same launch (2, 3 and 4 chunks; fewer outputs
+    than a tile), with a registered readout and without one."""
+    rng = W.SplitMix64(n)
+    body = [W.CX(q, q + d) for q in range(d)] + [W.CCX(0, 1, 2 * d)]
+    for k in range(cps):
+        a, b = rng.distinct(2 * d + 1, 2)
+        body += [W.CP(a, b, rng.angle())] + ([W.X(a), W.T(b)] if k % 5 == 4 else [])
+    gates = W.to_array([W.H(q) for q in range(d)] + body)
+    got, upd, fused = run(n, gates, 1 << d, FORCE, True)
+    assert fused, "the fused launch was not taken"
+    orc = OracleState(n)
+    orc.apply(gates, eps=EPS)
+    # |amplitude| = 2^(-d/2): a few roundings of 2^-53, and 4 of 2^-62 in the product
+    compare_states(got, orc.get(), EPS, atol=1e-14)
+    mask, value = ((1 << 9) - 1, 0), (0b101, 0)
+    st = sps.SparseState(n, 1 << d)
+    for o, v in FORCE + [(sps.SPS_OPT_READOUT_MIN_PLANES, 0)]:
+        st.set_option(o, v)
+    st.set_readout(mask, value)
+    st.reset()
+    st.apply(gates, EPS)
+    p = st.probability(mask, value)
+    assert st.counters().fused_readouts == 1
+    st.set_readout(None, None)
+    assert abs(p - st.probability(mask, value)) < 1e-14
+    st.close()
