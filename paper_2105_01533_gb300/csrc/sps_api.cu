@@ -253,6 +253,18 @@ void sps::hook_free(void* p, size_t bytes, void* stream) {
   f(ctx, p, (bytes + 255) & ~size_t(255), stream);
 }
 
+double* sps::device_view(const void* p, int device, bool host_too) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  const bool ok = (at.type == cudaMemoryTypeDevice && at.device == device) ||
+                  (host_too && at.type == cudaMemoryTypeHost);
+  if (!ok || (reinterpret_cast<uintptr_t>(at.devicePointer) & 7u)) return nullptr;
+  return static_cast<double*>(at.devicePointer);
+}
+
 namespace {
 
 LaunchCfg cfg_of(const sps_state* s) {
@@ -1510,12 +1522,26 @@ sps_status sps_nnz(sps_state* s, uint64_t* nnz) {
 sps_status sps_get_amplitudes(sps_state* s, uint64_t* key_hi, uint64_t* key_lo, double* re,
                               double* im, uint64_t cap, uint64_t* nnz_out) {
   if (!s || !key_lo || !re || !im || !nnz_out) return SPS_ERR_ARG;
-  sps_status st = sps_sync(s, nullptr);
+  // into device arrays one kernel copies the state before the one wait, which
+  // tells whether it did (see copy_entries)
+  const bool exported = device_view(key_lo, s->device, false) &&
+                        device_view(re, s->device, false) && device_view(im, s->device, false) &&
+                        (!key_hi || device_view(key_hi, s->device, false));
+  sps_status st = SPS_OK;
+  if (exported) {
+    st = flush_reset(s);
+    if (st != SPS_OK) return st;
+    if (launch_export(cfg_of(s), s->kw, s->ctl, s->bufs, key_hi, key_lo, re, im, cap,
+                      s->nnz_bound) < 0)
+      return cuda_ok(cudaGetLastError());
+    s->counters.kernel_launches += 1;
+  }
+  st = sps_sync(s, nullptr);
   if (st != SPS_OK) return st;
   const uint64_t n = s->ctl_host->nnz;
   *nnz_out = n;
   if (n > cap) return SPS_ERR_CAPACITY;
-  if (n == 0) return SPS_OK;
+  if (n == 0 || exported) return SPS_OK;
   const unsigned cur = s->ctl_host->cur;   // labels and amplitudes (Ctl::cur)
   SoA b = s->bufs.b[cur & 1u];
   b.re = s->bufs.b[(cur ^ (cur >> 1)) & 1u].re;
@@ -1657,14 +1683,11 @@ sps_status sps_probability(sps_state* s, const uint64_t mask[2], const uint64_t 
   const LaunchCfg lc = cfg_of(s);
   ProfScope ps(s, 12, s->pass_serial, 0, 0u);
   const int pn = launch_probability(lc, s->kw, s->ctl, s->bufs, mask[0], mask[1], value[0],
-                                    value[1], s->partials, prob_grid(s), s->dresult, ps.slot);
+                                    value[1], s->partials, prob_grid(s), s->hresult, ps.slot);
   ps.done();
   if (pn < 0) return cuda_ok(cudaGetLastError());
   s->counters.kernel_launches += 1;
-  if (cudaMemcpyAsync(s->hresult, s->dresult, sizeof(double), cudaMemcpyDeviceToHost, s->stream) !=
-      cudaSuccess)
-    return cuda_ok(cudaGetLastError());
-  st = cuda_ok(cudaStreamSynchronize(s->stream));
+  st = cuda_ok(cudaStreamSynchronize(s->stream));   // (hresult is pinned)
   if (st != SPS_OK) return st;
   *p = *s->hresult;
   return SPS_OK;
@@ -1683,12 +1706,16 @@ sps_status sps_probability_async(sps_state* s, const uint64_t mask[2], const uin
   const sps_status fs = flush_reset(s);
   if (fs != SPS_OK) return fs;
   const LaunchCfg lc = cfg_of(s);
+  // the kernel writes the caller's word itself where it can
+  double* direct = device_view(out, s->device, true);
   ProfScope ps(s, 12, s->pass_serial, 0, 0u);
   const int pn = launch_probability(lc, s->kw, s->ctl, s->bufs, mask[0], mask[1], value[0],
-                                    value[1], s->partials, prob_grid(s), s->dresult, ps.slot);
+                                    value[1], s->partials, prob_grid(s),
+                                    direct ? direct : s->dresult, ps.slot);
   ps.done();
   if (pn < 0) return cuda_ok(cudaGetLastError());
   s->counters.kernel_launches += 1;
+  if (direct) return SPS_OK;
   if (cudaMemcpyAsync(out, s->dresult, sizeof(double), cudaMemcpyDefault, s->stream) != cudaSuccess)
     return cuda_ok(cudaGetLastError());
   return SPS_OK;
@@ -1779,12 +1806,14 @@ sps_status sps_measure(sps_state* s, uint32_t qubit, double r, double* out) {
   const uint32_t serial = ++s->pass_serial;
   s->amp_force = true;   // the collapse moves labels
   ProfScope ps(s, 8, serial, 1, 1u);
+  double* direct = device_view(out, s->device, true);
   const int n = launch_measure(lc, s->kw, s->ctl, s->bufs, qubit, r, s->partials, s->prob_blocks,
-                               s->dmeasure, s->nnz_bound, s->masks.writer(), ps.slot);
+                               s->dmeasure, direct, s->nnz_bound, s->masks.writer(), ps.slot);
   ps.done();
   if (n < 0) return cuda_ok(cudaGetLastError());
   s->counters.kernel_launches += (uint64_t)n;
   s->counters.gates += 1;
+  if (direct) return SPS_OK;
   if (cudaMemcpyAsync(out, s->dmeasure, 2 * sizeof(double), cudaMemcpyDefault, s->stream) !=
       cudaSuccess)
     return cuda_ok(cudaGetLastError());

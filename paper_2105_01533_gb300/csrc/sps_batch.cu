@@ -551,6 +551,13 @@ sps_status sps_batch_get_amplitudes(sps_batch* b, uint32_t index, uint64_t* key_
   if (d.nnz > cap) return SPS_ERR_CAPACITY;
   if (d.nnz == 0) return SPS_OK;
   const unsigned c = d.cur;
+  if (device_view(key_lo, b->device, false) && device_view(re, b->device, false) &&
+      device_view(im, b->device, false) && (!key_hi || device_view(key_hi, b->device, false))) {
+    const SoA s{d.lo[c], d.kw == 2 ? d.hi[c] : nullptr, d.re[c], d.im[c]};
+    if (launch_copy_entries(b->stream, b->sms, s, d.nnz, key_hi, key_lo, re, im) < 0)
+      return cuda_st(cudaGetLastError());
+    return cuda_st(cudaStreamSynchronize(b->stream));
+  }
   const size_t bytes = 8 * d.nnz;
   bool ok = cudaMemcpyAsync(key_lo, d.lo[c], bytes, cudaMemcpyDefault, b->stream) == cudaSuccess &&
             cudaMemcpyAsync(re, d.re[c], bytes, cudaMemcpyDefault, b->stream) == cudaSuccess &&

@@ -593,10 +593,21 @@ struct ExpandLaunch {
 int launch_expand(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs, const ExpandLaunch& e,
                   uint64_t nnz_bound, unsigned long long* plog);
 // Measurement with collapse: partials holds 2 * nblocks doubles; res receives
-// {outcome, probability of the outcome, 1 / sqrt(p_outcome)}.
+// {outcome, probability of the outcome, 1 / sqrt(p_outcome)}, out (nullable,
+// memory the device can write) the first two.
 int launch_measure(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs, uint32_t qubit,
-                   double r, double* partials, int nblocks, double* res, uint64_t nnz_bound,
-                   uint32_t mg, unsigned long long* plog);
+                   double r, double* partials, int nblocks, double* res, double* out,
+                   uint64_t nnz_bound, uint32_t mg, unsigned long long* plog);
+// Copies the state to device arrays of at least cap entries (hi nullable), or
+// nothing if it has an error or more than cap entries.
+int launch_export(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs, uint64_t* hi,
+                  uint64_t* lo, double* re, double* im, uint64_t cap, uint64_t nnz_bound);
+// Copies n entries (s.hi null: high words 0) to device arrays (hi nullable).
+int launch_copy_entries(void* stream, int sms, SoA s, uint64_t n, uint64_t* hi, uint64_t* lo,
+                        double* re, double* im);
+// The address a kernel on `device` may write `words` doubles of the caller's at:
+// device memory of that device or pinned host memory, 8-byte aligned; else null.
+double* device_view(const void* p, int device, bool host_too);
 int launch_probability(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
                        uint64_t mask_lo, uint64_t mask_hi, uint64_t val_lo, uint64_t val_hi,
                        double* partials, int nblocks, double* result,
