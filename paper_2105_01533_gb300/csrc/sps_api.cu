@@ -1734,36 +1734,22 @@ sps_status sps_pauli_exp(sps_state* s, const uint64_t x[2], const uint64_t z[2],
   if (fs != SPS_OK) return fs;
   if ((x[0] | x[1]) == 0) {
     // A string of Z factors is diagonal: exp(-i t/2 P) multiplies a label by
-    // e^(-i t/2) or e^(i t/2) as the parity of its z bits is 0 or 1. A ladder of
-    // CNOTs puts that parity on the top z qubit, Rz(t) applies the phase, the
-    // ladder is undone: one fused run.
-    std::vector<uint32_t> bits;
-    for (uint32_t q = 0; q < s->nqubits; ++q)
-      if ((z[q >> 6] >> (q & 63)) & 1ull) bits.push_back(q);
-    const uint32_t t = bits.back();
-    std::vector<sps_gate> g;
-    auto rec = [&](uint8_t op, uint32_t tq, const uint64_t c[2], double th) {
-      sps_gate r;
-      std::memset(&r, 0, sizeof(r));
-      r.op = op;
-      r.t0 = (uint16_t)tq;
-      r.cmask[0] = c[0];
-      r.cmask[1] = c[1];
-      r.theta = th;
-      g.push_back(r);
-    };
-    for (size_t i = 0; i + 1 < bits.size(); ++i) {
-      const uint64_t c[2] = {bits[i] < 64 ? 1ull << bits[i] : 0ull,
-                             bits[i] >= 64 ? 1ull << (bits[i] - 64) : 0ull};
-      rec(SPS_OP_X, t, c, 0.0);
-    }
-    rec(SPS_OP_RZ, t, cmask, theta);
-    for (size_t i = bits.size() - 1; i-- > 0;) {
-      const uint64_t c[2] = {bits[i] < 64 ? 1ull << bits[i] : 0ull,
-                             bits[i] >= 64 ? 1ull << (bits[i] - 64) : 0ull};
-      rec(SPS_OP_X, t, c, 0.0);
-    }
-    return sps_apply(s, g.data(), g.size(), prune_eps, nullptr);
+    // e^(-i t/2) or e^(i t/2) as the parity of its z bits is 0 or 1. It counts as
+    // the run it stands for: a ladder of CNOTs that puts the parity on one z
+    // qubit, Rz(t) there, the ladder undone.
+    const uint32_t bits =
+        (uint32_t)(__builtin_popcountll(z[0]) + __builtin_popcountll(z[1]));
+    const uint32_t ngates = 2 * bits - 1;
+    ++s->apply_serial;
+    ProfScope ps(s, 1, ++s->pass_serial, ngates, 2u);
+    const int n = launch_zphase(cfg_of(s), s->kw, s->ctl, s->bufs, z, cmask, std::cos(0.5 * theta),
+                                std::sin(0.5 * theta), ngates, s->nnz_bound, ps.slot);
+    ps.done();
+    if (n < 0) return cuda_ok(cudaGetLastError());
+    s->counters.kernel_launches += 1;
+    s->counters.fused_passes += 1;
+    s->counters.gates += ngates;
+    return SPS_OK;
   }
   BranchOp op;
   std::memset(&op, 0, sizeof(op));

@@ -603,8 +603,13 @@ int launch_measure(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs, uint
 int launch_export(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs, uint64_t* hi,
                   uint64_t* lo, double* re, double* im, uint64_t cap, uint64_t nnz_bound);
 // Copies n entries (s.hi null: high words 0) to device arrays (hi nullable).
-int launch_copy_entries(void* stream, int sms, SoA s, uint64_t n, uint64_t* hi, uint64_t* lo,
-                        double* re, double* im);
+int launch_copy_entries(void* stream, SoA s, uint64_t n, uint64_t* hi, uint64_t* lo, double* re,
+                        double* im);
+// exp(-i t/2 P) of a string P of Z factors (bits z, controls c; cs, sn = cos, sin
+// of t/2), counted as ngates gates.
+int launch_zphase(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs, const uint64_t z[2],
+                  const uint64_t c[2], double cs, double sn, uint32_t ngates, uint64_t nnz_bound,
+                  unsigned long long* plog);
 // The address a kernel on `device` may write `words` doubles of the caller's at:
 // device memory of that device or pinned host memory, 8-byte aligned; else null.
 double* device_view(const void* p, int device, bool host_too);

@@ -123,6 +123,44 @@ __global__ void __launch_bounds__(256) k_fused(Ctl* ctl, Bufs bufs, const FusedA
 }
 
 // ---------------------------------------------------------------------------
+// A Pauli exponential of Z factors only: a label's amplitude times
+// cos(t/2) - i sin(t/2) or its conjugate as the parity of its z bits is even or
+// odd, where its controls are set. Bounded by the launch below some 100,000
+// entries (134,596: 4 us), then by the amplitudes' bytes and the products. As a run of
+// CNOTs, Rz and CNOTs, compiled and uploaded on every call, it took 7.3 us and an
+// upload that the stream waited for.
+struct ZArgs {
+  uint64_t z[2], c[2];
+  double cs, sn;
+  uint32_t ngates;   // gates of that run (the update count)
+};
+
+template <int KW>
+__global__ void __launch_bounds__(256) k_zphase(Ctl* ctl, Bufs bufs, const ZArgs a,
+                                                unsigned long long* plog) {
+  const uint64_t n = ctl->nnz;
+  if (plog && blockIdx.x == 0 && threadIdx.x == 0) {
+    plog[0] = n;
+    plog[1] = n;
+  }
+  if (ctl->status != 0u) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) ctl->updates += n * a.ngates;
+  const SoA s = pick(bufs, ctl->cur);
+  const bool read_hi = KW == 2 && (a.z[1] | a.c[1]) != 0ull;
+  const bool read_lo = (a.z[0] | a.c[0]) != 0ull;
+  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
+       i += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t k0 = read_lo ? s.lo[i] : 0ull, k1 = read_hi ? s.hi[i] : 0ull;
+    if ((k0 & a.c[0]) != a.c[0] || (k1 & a.c[1]) != a.c[1]) continue;
+    double re = s.re[i], im = s.im[i];
+    const bool odd = ((__popcll(k0 & a.z[0]) + __popcll(k1 & a.z[1])) & 1) != 0;
+    cmul_rn(re, im, a.cs, odd ? a.sn : -a.sn);
+    s.re[i] = re;
+    s.im[i] = im;
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Bit-sliced fused pass. A warp owns a tile of G groups x 32 entries:
 //   1. load: 32 entries at a time; each 32-bit label word the pass needs is
 //      transposed across the warp (shuffle butterfly), so lane j holds
@@ -981,8 +1019,8 @@ __global__ void __launch_bounds__(256) k_probability(Ctl* ctl, Bufs bufs, uint64
 // the control block, then the copies, then another wait. 65,536 entries with
 // what leads up to it 156 -> 137 us, 256 circuits' states 5.4 -> 2.9 ms; 537 MB
 // go as fast as with the copy engine (20 us less a pass: one wait less).
-// One array of n words (src null: zeros) by the whole grid, 16 bytes an access and
-// four in flight a thread where both ends are aligned for it.
+// One array of n words (src null: zeros) by a row of blocks, 16 bytes an access
+// and four in flight a thread where both ends are aligned for it.
 __device__ __forceinline__ void copy_words(const uint64_t* src, uint64_t* dst, uint64_t n) {
   const uint64_t tid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -1005,14 +1043,16 @@ __device__ __forceinline__ void copy_words(const uint64_t* src, uint64_t* dst, u
   if ((n & 1ull) != 0ull && tid == 0) dst[n - 1] = src ? src[n - 1] : 0ull;
 }
 
-// (array after array: what the last pass wrote is in L2 and is read first while
-// it still is; all arrays side by side took 354 us for 338 on a pass of 5 M entries)
+// Row blockIdx.y of the grid copies one array. Rows start in order, so what the
+// last pass wrote is read first, while it is in L2 (all arrays side by side
+// took 354 us for 338 on a pass of 5 M entries); few entries go in one wave.
 __device__ __forceinline__ void copy_entries(const SoA& s, uint64_t n, uint64_t* hi, uint64_t* lo,
                                              double* re, double* im) {
-  copy_words(s.lo, lo, n);
-  if (hi) copy_words(s.hi, hi, n);
-  copy_words(reinterpret_cast<const uint64_t*>(s.re), reinterpret_cast<uint64_t*>(re), n);
-  copy_words(reinterpret_cast<const uint64_t*>(s.im), reinterpret_cast<uint64_t*>(im), n);
+  const unsigned y = blockIdx.y;
+  if (y == 0) copy_words(s.lo, lo, n);
+  else if (y == 1) copy_words(reinterpret_cast<const uint64_t*>(s.re), reinterpret_cast<uint64_t*>(re), n);
+  else if (y == 2) copy_words(reinterpret_cast<const uint64_t*>(s.im), reinterpret_cast<uint64_t*>(im), n);
+  else copy_words(s.hi, hi, n);
 }
 
 // The state, if it has no error and fits cap (the host finds either out from
@@ -1549,19 +1589,36 @@ int launch_measure(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs, uint
   return cudaPeekAtLastError() == cudaSuccess ? 2 : -1;
 }
 
+// Blocks of 256 threads a row, eight words a thread; at most about a resident wave
+// (the bound may be far above the count, and rows still start in order).
+static dim3 copy_grid(uint64_t n, bool hi) {
+  const uint64_t b = (n + 2047) / 2048;
+  return dim3((unsigned)(b < 1 ? 1 : b > 1024 ? 1024 : b), hi ? 4u : 3u);
+}
+
 int launch_export(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs, uint64_t* hi,
                   uint64_t* lo, double* re, double* im, uint64_t cap, uint64_t nnz_bound) {
-  const int blocks = grid_for((nnz_bound + 1) / 2, 256, lc.max_blocks);
+  const dim3 grid = copy_grid(nnz_bound, hi != nullptr);
   cudaStream_t st = (cudaStream_t)lc.stream;
-  if (key_words == 1) k_export<1><<<blocks, 256, 0, st>>>(ctl, bufs, hi, lo, re, im, cap);
-  else k_export<2><<<blocks, 256, 0, st>>>(ctl, bufs, hi, lo, re, im, cap);
+  if (key_words == 1) k_export<1><<<grid, 256, 0, st>>>(ctl, bufs, hi, lo, re, im, cap);
+  else k_export<2><<<grid, 256, 0, st>>>(ctl, bufs, hi, lo, re, im, cap);
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 
-int launch_copy_entries(void* stream, int sms, SoA s, uint64_t n, uint64_t* hi, uint64_t* lo,
-                        double* re, double* im) {
-  const int blocks = grid_for((n + 1) / 2, 256, 8 * (sms > 0 ? sms : 1));
-  k_copy_entries<<<blocks, 256, 0, (cudaStream_t)stream>>>(s, n, hi, lo, re, im);
+int launch_copy_entries(void* stream, SoA s, uint64_t n, uint64_t* hi, uint64_t* lo, double* re,
+                        double* im) {
+  k_copy_entries<<<copy_grid(n, hi != nullptr), 256, 0, (cudaStream_t)stream>>>(s, n, hi, lo, re, im);
+  return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
+}
+
+int launch_zphase(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs, const uint64_t z[2],
+                  const uint64_t c[2], double cs, double sn, uint32_t ngates, uint64_t nnz_bound,
+                  unsigned long long* plog) {
+  const ZArgs a{{z[0], z[1]}, {c[0], c[1]}, cs, sn, ngates};
+  const int blocks = grid_for(nnz_bound, lc.threads, lc.max_blocks);
+  cudaStream_t st = (cudaStream_t)lc.stream;
+  if (key_words == 1) k_zphase<1><<<blocks, lc.threads, 0, st>>>(ctl, bufs, a, plog);
+  else k_zphase<2><<<blocks, lc.threads, 0, st>>>(ctl, bufs, a, plog);
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 
