@@ -1315,6 +1315,40 @@ __device__ __forceinline__ void amp_round(const AmpArgs& a, const AmpGate* sg, c
   }
 }
 
+// The writers left in the queues of a block's warps after its last chunk, put
+// together by class, so a class leaves one partial round a block instead of one
+// a warp (a round lasts as long with one group as with all). Every thread of
+// the block calls leftover_gather; a warp then runs rounds warp, warp + warps ...
+// of leftover_rounds(c). With 8 chunks a warp (635,376 entries) partial rounds
+// were up to five of thirteen.
+struct AmpLeft {
+  uint32_t count[kAmpMaxActive];               // writers of class c + 1
+  uint32_t idx[kAmpMaxActive][8 * 32];         // (a warp leaves fewer than 32)
+  uint32_t act[kAmpMaxActive][8 * 32];
+};
+
+__device__ __forceinline__ void leftover_gather(AmpLeft& l, const uint32_t (*sqi)[kAmpRing],
+                                                const uint32_t (*sqa)[kAmpRing],
+                                                const uint32_t (&head)[kAmpMaxActive],
+                                                const uint32_t (&tail)[kAmpMaxActive],
+                                                unsigned lane) {
+  if (threadIdx.x < kAmpMaxActive) l.count[threadIdx.x] = 0u;
+  __syncthreads();
+#pragma unroll
+  for (uint32_t c = 0; c < kAmpMaxActive; ++c) {
+    const uint32_t left = tail[c] - head[c];
+    if (left == 0u) continue;
+    uint32_t at = 0u;
+    if (lane == 0) at = atomicAdd(&l.count[c], left);
+    at = __shfl_sync(FULL, at, 0);
+    if (lane < left) {
+      l.idx[c][at + lane] = sqi[c][(head[c] + lane) % kAmpRing];
+      l.act[c][at + lane] = sqa[c][(head[c] + lane) % kAmpRing];
+    }
+  }
+  __syncthreads();
+}
+
 // One warp per chunk of 32 entries (chunks handed out by a counter), no block
 // barrier inside the loop:
 //   1. the chunk's labels as bit-planes in the warp's shared rows; lane j
@@ -1336,6 +1370,7 @@ __global__ void __launch_bounds__(256, SPS_AMP_MIN_BLOCKS) k_amp_layer(Ctl* ctl,
   __shared__ uint64_t spar[2 * kMaxAmpParity];     // sign conditions (AMP_PARITY)
   __shared__ uint32_t sqi[8][kAmpMaxActive][kAmpRing];   // per warp and class: writers' indices
   __shared__ uint32_t sqa[8][kAmpMaxActive][kAmpRing];   // and their active gates
+  __shared__ AmpLeft left;
   extern __shared__ uint4 fsm[];                   // AMP_WALK: the phase run's op stream
   const bool go = ctl->amp_go != 0u;
   LabelMasks lm{};
@@ -1433,15 +1468,16 @@ __global__ void __launch_bounds__(256, SPS_AMP_MIN_BLOCKS) k_amp_layer(Ctl* ctl,
       if (__any_sync(FULL, bad)) break;   // the attempt fails: the usual passes run
       ch = __shfl_sync(FULL, next, 0);
     }
-    // the partial rounds left in the queues
-    if (!__any_sync(FULL, bad)) {
+    // the writers left in the block's queues
+    if (!__syncthreads_or(bad ? 1 : 0)) {
+      leftover_gather(left, sqi[warp], sqa[warp], qhead, qtail, lane);
 #pragma unroll
       for (uint32_t c = 1; c <= kAmpMaxActive; ++c) {
-        const uint32_t left = qtail[c - 1] - qhead[c - 1];
-        if (left)
+        const uint32_t per = 32u >> (c < 5u ? c : 5u), have = left.count[c - 1];
+        for (uint32_t g = warp * per; g < have; g += (blockDim.x >> 5) * per)
           amp_round<KW, REAL, POST>(a, sg, spar, pl, fsm, s, out, itab, mask, ep, eps_bits, c,
-                                    sqi[warp][c - 1], sqa[warp][c - 1], qhead[c - 1], left, lane,
-                                    bad, written, hic);
+                                    left.idx[c - 1] + g, left.act[c - 1] + g, 0u,
+                                    have - g < per ? have - g : per, lane, bad, written, hic);
       }
     }
     // every entry written exactly once, or some group had no writer
@@ -1769,7 +1805,8 @@ __device__ __forceinline__ void grp_round(GrpCtl* g, const GrpArgs& a, const Amp
 template <int KW>
 __device__ __forceinline__ void grp_emit(GrpCtl* g, const GrpArgs& a, const AmpGate* sg,
                                          uint32_t* pl, uint32_t (*sqi)[kAmpRing],
-                                         uint32_t (*sqa)[kAmpRing], const SoA& s, const SoA& out,
+                                         uint32_t (*sqa)[kAmpRing], AmpLeft& left, const SoA& s,
+                                         const SoA& out,
                                          uint64_t n, uint64_t entries,
                                          const unsigned long long* itab, uint64_t mask,
                                          unsigned long long ep) {
@@ -1829,12 +1866,14 @@ __device__ __forceinline__ void grp_emit(GrpCtl* g, const GrpArgs& a, const AmpG
     }
     ch = __shfl_sync(FULL, next, 0);
   }
+  leftover_gather(left, sqi, sqa, qhead, qtail, lane);
+  const unsigned warp = threadIdx.x >> 5;
 #pragma unroll
   for (uint32_t c = 1; c <= kAmpMaxActive; ++c) {
-    const uint32_t left = qtail[c - 1] - qhead[c - 1];
-    if (left)
-      grp_round<KW>(g, a, sg, s, out, n, itab, mask, ep, eps_bits, c, sqi[c - 1], sqa[c - 1],
-                    qhead[c - 1], left, lane, sum);
+    const uint32_t per = 32u >> (c < 5u ? c : 5u), have = left.count[c - 1];
+    for (uint32_t f = warp * per; f < have; f += (blockDim.x >> 5) * per)
+      grp_round<KW>(g, a, sg, s, out, n, itab, mask, ep, eps_bits, c, left.idx[c - 1] + f,
+                    left.act[c - 1] + f, 0u, have - f < per ? have - f : per, lane, sum);
   }
   merge_label_masks(g->lm[blockIdx.x % kMaskStripes], sum.mo0, sum.mo1, sum.ma0, sum.ma1);
   for (int dd = 16; dd > 0; dd >>= 1) {
@@ -1978,6 +2017,7 @@ __device__ __forceinline__ bool chain_groups(Ctl* ctl, Bufs bufs, unsigned long 
   __shared__ uint32_t splanes[8][128];
   __shared__ uint32_t sqi[8][kAmpMaxActive][kAmpRing];
   __shared__ uint32_t sqa[8][kAmpMaxActive][kAmpRing];
+  __shared__ AmpLeft left;
   if (__syncthreads_or(ctl->status != 0u)) return false;
   const GrpArgs& ga = a.grp;
   const unsigned warp = threadIdx.x >> 5;
@@ -2008,7 +2048,8 @@ __device__ __forceinline__ bool chain_groups(Ctl* ctl, Bufs bufs, unsigned long 
   if (__ldcg(&g->bad) != 0u) return false;
   const uint64_t all = n + __ldcg(&g->grown);
   const uint64_t entries = all < ga.capacity ? all : ga.capacity;
-  grp_emit<KW>(g, ga, sg, splanes[warp], sqi[warp], sqa[warp], s, out, n, entries, itab, mask, ep);
+  grp_emit<KW>(g, ga, sg, splanes[warp], sqi[warp], sqa[warp], left, s, out, n, entries, itab,
+               mask, ep);
   grid_barrier(ctl, serial, tag);
   if (blockIdx.x == 0 && threadIdx.x < 32) {
     // every intermediate state fits if every member of every group does
