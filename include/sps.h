@@ -229,7 +229,8 @@ sps_status sps_measure(sps_state* s, uint32_t qubit, double r, double* out);
 
 /* Tuning options (see sps_set_option). */
 typedef enum sps_option {
-  SPS_OPT_LOAD_FACTOR_PCT = 1, /* target branching-table load, 10..90 (default 50) */
+  SPS_OPT_LOAD_FACTOR_PCT = 1, /* target branching-table load, 10..90 (default 50); the
+                                  gather index may take half of it up to 32 MB */
   SPS_OPT_PROBE_LIMIT = 2,     /* max slots probed per insert, >= 1 (default: table size) */
   SPS_OPT_BLOCK_THREADS = 3,   /* threads per block of the per-element kernels: 128 or
                                   256 (default 256) */

