@@ -559,10 +559,10 @@ sps_status sps_create(uint32_t nqubits, uint64_t capacity, void* cuda_stream, sp
   s->itab_log2 = table_log2_for((capacity + 1) / 2, 50, 40);
   if ((st = dev_alloc(s, (sizeof(unsigned long long) << s->itab_log2), &p)) != SPS_OK) return fail(st);
   s->itab = (unsigned long long*)p;
-  if ((st = dev_alloc(s, sizeof(Ctl), &p)) != SPS_OK) return fail(st);
+  const size_t ctl_bytes = (sizeof(Ctl) + 255) & ~size_t(255);
+  if ((st = dev_alloc(s, ctl_bytes + sizeof(GrpCtl), &p)) != SPS_OK) return fail(st);
   s->ctl = (Ctl*)p;
-  if ((st = dev_alloc(s, sizeof(GrpCtl), &p)) != SPS_OK) return fail(st);
-  s->grp = (GrpCtl*)p;
+  s->grp = (GrpCtl*)((unsigned char*)p + ctl_bytes);
   // partials: 2 per block (the measurement's two sums), then the probability
   // result and the measurement's three results
   if ((st = dev_alloc(s, sizeof(double) * (2 * s->prob_blocks + 4), &p)) != SPS_OK) return fail(st);
@@ -919,7 +919,7 @@ static sps_status build_plan(sps_state* s, const sps_gate* gates, size_t ngates,
     ngates = rewritten.size();
   }
   const sps_status cs = compile(gates, ngates, s->nqubits, s->max_fused_ops, &P->passes, bad,
-                                &P->kb_out, s->expand, s->fold, s->layer_max);
+                                &P->kb_out, s->expand, s->fold, s->layer_max, false);
   if (cs != SPS_OK) return cs;
   // layers that a one-block run would take go back to one pass per gate (the
   // one-block engine runs passes, the layer kernels are whole-GPU)
@@ -1112,6 +1112,12 @@ static sps_status build_plan(sps_state* s, const sps_gate* gates, size_t ngates,
       }
     }
     ++i;
+  }
+  // the op streams of the fused passes that are not bit-sliced
+  for (size_t i = 0; i < np;) {
+    const size_t end = P->seg_end[i] ? P->seg_end[i] : i + 1;
+    for (; i < end; ++i)
+      if (P->passes[i].kind == PASS_FUSED && P->bs[i].ops.empty()) encode_ops(&P->passes[i]);
   }
   // an expansion from |0...0> and the bit-sliced run after it, as one launch
   // (taken at apply time when the reset is still pending)

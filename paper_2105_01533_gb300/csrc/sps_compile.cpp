@@ -455,7 +455,7 @@ sps_status commute_gates(const sps_gate* gates, size_t ngates, uint32_t nqubits,
 
 sps_status compile(const sps_gate* gates, size_t ngates, uint32_t nqubits,
                    uint32_t max_fused_ops, std::vector<Pass>* out, size_t* bad, KnownBits* kb,
-                   bool expand, bool fold, uint32_t layer_max) {
+                   bool expand, bool fold, uint32_t layer_max, bool encode) {
   if (layer_max > kMaxLayerGates) layer_max = kMaxLayerGates;
   if (max_fused_ops == 0 || max_fused_ops > kMaxFusedOps) max_fused_ops = kDefaultMaxFusedOps;
   out->clear();
@@ -551,7 +551,13 @@ sps_status compile(const sps_gate* gates, size_t ngates, uint32_t nqubits,
   }
   close_run();
   for (Pass& p : *out) {
-    if (p.kind == PASS_FUSED) encode_ops(&p);
+    if (p.kind == PASS_FUSED) {
+      for (const FOp& o : p.ops) {
+        p.has_perm = p.has_perm || (o.kind & FOP_FLIP);
+        p.has_phase = p.has_phase || (o.kind & (FOP_CNT | FOP_PH));
+      }
+      if (encode) encode_ops(&p);
+    }
     if (p.kind == PASS_EXPAND) build_expand(&p);
   }
   if (kb) *kb = k;
@@ -562,7 +568,6 @@ void encode_ops(Pass* p) {
   const std::vector<FOp>& ops = p->ops;
   std::vector<OpWord>* words = &p->words;
   words->clear();
-  p->has_perm = p->has_phase = false;
   // the ops split into flips and phase ops, each with its level
   struct Prim {
     uint64_t c[2], t[2];
@@ -599,8 +604,6 @@ void encode_ops(Pass* p) {
   // fire slots in op order; slot k's factor is the phase its op applies
   std::vector<double> factor;
   for (const FOp& o : ops) {
-    p->has_perm = p->has_perm || (o.kind & FOP_FLIP);
-    p->has_phase = p->has_phase || (o.kind & (FOP_CNT | FOP_PH));
     uint64_t w0 = (uint64_t)(o.a0 & 7u) << kOpCountShift;
     uint64_t w1 = (uint64_t)(o.a1 & 7u) << kOpCountShift;
     if (o.ph != NO_PH) {

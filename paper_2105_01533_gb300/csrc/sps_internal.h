@@ -316,10 +316,12 @@ sps_status commute_gates(const sps_gate* gates, size_t ngates, uint32_t nqubits,
 // gates (updating *kb on success); if expand it forms expansion passes, if
 // fold it resolves known qubits in fused runs (lower_known).
 // layer_max > 1 groups consecutive disjoint branching gates into layer passes.
+// encode: the fused passes' op streams too (else the caller's, encode_ops: a pass
+// that runs bit-sliced needs none).
 sps_status compile(const sps_gate* gates, size_t ngates, uint32_t nqubits,
                    uint32_t max_fused_ops, std::vector<Pass>* out, size_t* bad,
                    KnownBits* kb = nullptr, bool expand = false, bool fold = false,
-                   uint32_t layer_max = 1);
+                   uint32_t layer_max = 1, bool encode = true);
 // The most nonzeros a state can reach from |0...0> through the passes (every
 // branching gate at most doubles the count), capped at the capacity.
 uint64_t projected_peak(const std::vector<Pass>& passes, uint64_t capacity);
