@@ -65,8 +65,7 @@ __device__ __forceinline__ void carry_label_masks(Ctl* ctl, uint32_t mg) {
 // Up to 32 MB, and where the state has the room, it is twice that: a build and a
 // lookup wait for the longest probe of a warp, and the table stays in L2 (labels
 // and slots of 134,596 entries: a step of 24 Pauli strings 1,249 -> 1,116 us; of
-// 40,000 to 800,000: 45 branching gates 2,263 -> 2,113 us; in DRAM the larger
-// table would cost more sectors than it saves).
+// 40,000 to 800,000: 45 branching gates 2,263 -> 2,113 us).
 constexpr uint32_t kIdxRoomyLog2 = 22;
 
 __device__ __forceinline__ uint64_t itab_mask(uint64_t n, uint32_t load_pct, uint32_t max_log2) {
@@ -122,10 +121,10 @@ __device__ __forceinline__ uint64_t idx_entry(const IdxBucket& k, uint32_t t) {
 // a word of this epoch that comes back is carried on to the next slot (every
 // slot it passes stays taken, so lookups find it). The four labels' loads are
 // in flight together, and so is each round of their claims. What bounds it is
-// the longest of a warp's chains: with a load and a compare-and-swap a claim,
-// one label after the other, 457,728 labels on 2^20 slots took 32 us, with the
-// bucket loaded first and its first free slot swapped 54 (half the claims lost
-// a race), now 18.
+// the longest of a warp's chains. 780,000 labels: with a load and a
+// compare-and-swap a claim, one label after the other, 41 us; with the bucket
+// loaded first and its first free slot swapped, 83 (half the claims lost a
+// race); with an atomic maximum a slot, one label after the other, 57; now 31.
 // Returns false in the threads that found the table full.
 template <int KW, typename Want>
 __device__ __forceinline__ bool idx_build(unsigned long long* itab, uint64_t mask,
@@ -210,49 +209,6 @@ __device__ __forceinline__ uint64_t idx_find(const unsigned long long* itab, uin
   return ~0ull;
 }
 
-// U lookups of one lane at once, bucket loads in flight together, then the
-// candidates' labels and amplitudes; the few that a bucket does not decide (it
-// is full, or its candidate is another label) go through idx_find.
-template <int KW, int U>
-__device__ __forceinline__ void idx_find_n(const unsigned long long* itab, uint64_t mask,
-                                           unsigned long long ep, const SoA& s,
-                                           const bool (&want)[U], const uint64_t (&lo)[U],
-                                           const uint64_t (&hi)[U], bool (&found)[U],
-                                           double (&re)[U], double (&im)[U]) {
-  uint32_t m[U];
-  uint64_t j[U], l0[U], l1[U];
-  IdxBucket k[U];
-  unsigned long long fp[U];
-#pragma unroll
-  for (int u = 0; u < U; ++u) {
-    found[u] = false;
-    re[u] = im[u] = 0.0;
-    if (!want[u]) continue;
-    const uint64_t hv = hash_label<KW>(lo[u], hi[u]);
-    fp[u] = idx_print(hv);
-    k[u] = idx_load(itab, hv & mask & ~3ull);
-  }
-#pragma unroll
-  for (int u = 0; u < U; ++u) {
-    m[u] = want[u] ? idx_match(k[u], ep, fp[u]) : 16u;
-    if ((m[u] & 15u) == 0u) continue;
-    j[u] = idx_entry(k[u], (uint32_t)__ffs(m[u]) - 1u);
-    l0[u] = s.lo[j[u]];
-    l1[u] = KW == 2 ? s.hi[j[u]] : 0ull;
-    re[u] = s.re[j[u]];
-    im[u] = s.im[j[u]];
-  }
-#pragma unroll
-  for (int u = 0; u < U; ++u) {
-    if (m[u] == 16u) continue;
-    found[u] = (m[u] & 15u) != 0u && l0[u] == lo[u] && (KW == 1 || l1[u] == hi[u]);
-    if (!found[u]) {
-      re[u] = im[u] = 0.0;
-      found[u] = idx_find<KW, true>(itab, mask, ep, s, lo[u], hi[u], &re[u], &im[u]) != ~0ull;
-    }
-  }
-}
-
 template <int KW>
 __device__ __forceinline__ void gather_build(Ctl* ctl, Bufs bufs, unsigned long long* itab,
                                              const GatherArgs& a, unsigned long long* plog) {
@@ -324,9 +280,10 @@ __device__ __forceinline__ void own_rows(const BranchOp& op, bool x, bool found,
   }
 }
 
-// U entries a thread and step (blockDim apart): their lookups overlap, and a
-// step takes its output places with one atomic for U * blockDim entries.
-template <int KW, int U>
+// One entry a thread and step. (Two, their lookups in flight together, took
+// longer at every size: 134,596 entries 15.8 and 15.9 us, 300,000 24 and 28, 1 M
+// 53 and 59, 4 M 217 and 274: the registers cost more resident warps.)
+template <int KW>
 __device__ __forceinline__ void gather_emit(Ctl* ctl, Bufs bufs, const unsigned long long* itab,
                                             const GatherArgs& a, unsigned long long* plog) {
   __shared__ unsigned warp_cnt[2][32];
@@ -355,41 +312,28 @@ __device__ __forceinline__ void gather_emit(Ctl* ctl, Bufs bufs, const unsigned 
   if (blockIdx.x == 0 && threadIdx.x == 0) reset_label_masks(ctl, mg_rs(a.mg));
   uint64_t mo0 = 0, mo1 = 0, ma0 = ~0ull, ma1 = ~0ull;   // OR / AND of the written labels
   unsigned side = 0;   // which half of the shared words this step uses
-  for (uint64_t base = (uint64_t)U * blockIdx.x * blockDim.x; base < n;
-       base += (uint64_t)U * gridDim.x * blockDim.x, side ^= 1u) {
-    uint64_t k0[U], k1[U], p0[U], p1[U];
-    double re[U], im[U], pr[U], pi[U];
-    bool act[U], look[U], found[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const uint64_t i = base + (uint64_t)u * blockDim.x + threadIdx.x;
-      const bool valid = i < n;
-      k0[u] = valid ? s.lo[i] : 0ull;
-      k1[u] = (KW == 2 && valid) ? s.hi[i] : 0ull;
-      re[u] = valid ? s.re[i] : 0.0;   // (a zero is pruned: nothing past the end is written)
-      im[u] = valid ? s.im[i] : 0.0;
-      act[u] = valid && (k0[u] & op.c[0]) == op.c[0] && (k1[u] & op.c[1]) == op.c[1];
-      if (op.givens)
-        act[u] = act[u] && (label_bit(k0[u], k1[u], op.sbit) != label_bit(k0[u], k1[u], op.qbit));
-      p0[u] = k0[u] ^ op.m[0];
-      p1[u] = k1[u] ^ op.m[1];
-      look[u] = act[u] && !no_partners;
+  for (uint64_t base = blockIdx.x * (uint64_t)blockDim.x; base < n;
+       base += (uint64_t)gridDim.x * blockDim.x, side ^= 1u) {
+    const uint64_t i = base + threadIdx.x;
+    const bool valid = i < n;
+    const uint64_t k0 = valid ? s.lo[i] : 0ull;
+    const uint64_t k1 = (KW == 2 && valid) ? s.hi[i] : 0ull;
+    double vr = valid ? s.re[i] : 0.0;   // (a zero is pruned: nothing past the end is written)
+    double vi = valid ? s.im[i] : 0.0;
+    const uint64_t p0 = k0 ^ op.m[0], p1 = k1 ^ op.m[1];
+    double qr = 0.0, qi = 0.0;
+    bool act = valid && (k0 & op.c[0]) == op.c[0] && (k1 & op.c[1]) == op.c[1];
+    if (op.givens) act = act && (label_bit(k0, k1, op.sbit) != label_bit(k0, k1, op.qbit));
+    if (act) {
+      double pr = 0.0, pi = 0.0;
+      const bool found =
+          !no_partners && idx_find<KW, true>(itab, mask, ep, s, p0, p1, &pr, &pi) != ~0ull;
+      const double re = vr, im = vi;
+      own_rows(op, label_bit(k0, k1, op.sbit), found, k0, k1, re, im, pr, pi, &vr, &vi, &qr, &qi);
     }
-    idx_find_n<KW, U>(itab, mask, ep, s, look, p0, p1, found, pr, pi);
-    double vr[U], vi[U], qr[U], qi[U];
-    unsigned bo[U], bq[U], cnt = 0u;
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      vr[u] = re[u];
-      vi[u] = im[u];
-      qr[u] = qi[u] = 0.0;
-      if (act[u])
-        own_rows(op, label_bit(k0[u], k1[u], op.sbit), found[u], k0[u], k1[u], re[u], im[u], pr[u],
-                 pi[u], &vr[u], &vi[u], &qr[u], &qi[u]);
-      bo[u] = __ballot_sync(FULL, keep_amp(vr[u], vi[u], a.eps2, eps_bits));
-      bq[u] = __ballot_sync(FULL, keep_amp(qr[u], qi[u], a.eps2, eps_bits));
-      cnt += __popc(bo[u]) + __popc(bq[u]);
-    }
+    const unsigned bo = __ballot_sync(FULL, keep_amp(vr, vi, a.eps2, eps_bits));
+    const unsigned bq = __ballot_sync(FULL, keep_amp(qr, qi, a.eps2, eps_bits));
+    const unsigned cnt = __popc(bo) + __popc(bq);
     if (lane == 0) warp_cnt[side][warp] = cnt;
     __syncthreads();
     if (warp == 0) {
@@ -422,11 +366,8 @@ __device__ __forceinline__ void gather_emit(Ctl* ctl, Bufs bufs, const unsigned 
       }
       pos += __popc(b);
     };
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      put(bo[u], k0[u], k1[u], vr[u], vi[u]);
-      put(bq[u], p0[u], p1[u], qr[u], qi[u]);
-    }
+    put(bo, k0, k1, vr, vi);
+    put(bq, p0, p1, qr, qi);
   }
   merge_label_masks(ctl, mg_wr(a.mg), mo0, mo1, ma0, ma1);
   if (threadIdx.x == 0) {
@@ -465,12 +406,12 @@ __global__ void __launch_bounds__(256) k_gather_build(Ctl* ctl, Bufs bufs, unsig
   gather_build<KW>(ctl, bufs, itab, a, plog);
 }
 
-template <int KW, int U>
+template <int KW>
 __global__ void __launch_bounds__(256) k_gather_emit(Ctl* ctl, Bufs bufs,
                                                      const unsigned long long* itab,
                                                      const __grid_constant__ GatherArgs a,
                                                      unsigned long long* plog) {
-  gather_emit<KW, U>(ctl, bufs, itab, a, plog);
+  gather_emit<KW>(ctl, bufs, itab, a, plog);
 }
 
 // ---------------------------------------------------------------------------
@@ -2131,7 +2072,7 @@ __global__ void __launch_bounds__(256) k_chain(Ctl* ctl, Bufs bufs, unsigned lon
     } else {
       gather_build<KW>(ctl, bufs, itab, st.g, nullptr);
       grid_barrier(ctl, serial, tag);
-      gather_emit<KW, 2>(ctl, bufs, itab, st.g, nullptr);
+      gather_emit<KW>(ctl, bufs, itab, st.g, nullptr);
     }
     // (nothing of this launch reads the last pass's state, unless ...)
     if (k + 1u < a.nsteps || a.w.ngates || plog) grid_barrier(ctl, serial, tag);
@@ -2426,15 +2367,10 @@ int launch_gather_part(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
     else
       k_gather_build<2><<<blocks, lc.threads, 0, st>>>(ctl, bufs, itab, a, plog);
   } else {
-    const int u = nnz_bound > (uint64_t)lc.max_blocks * (uint64_t)lc.threads ? 2 : 1;
-    const int eb = grid_of((nnz_bound + u - 1) / u, lc.threads, lc.max_blocks);
-    if (key_words == 1) {
-      if (u == 1) k_gather_emit<1, 1><<<eb, lc.threads, 0, st>>>(ctl, bufs, itab, a, plog);
-      else k_gather_emit<1, 2><<<eb, lc.threads, 0, st>>>(ctl, bufs, itab, a, plog);
-    } else {
-      if (u == 1) k_gather_emit<2, 1><<<eb, lc.threads, 0, st>>>(ctl, bufs, itab, a, plog);
-      else k_gather_emit<2, 2><<<eb, lc.threads, 0, st>>>(ctl, bufs, itab, a, plog);
-    }
+    if (key_words == 1)
+      k_gather_emit<1><<<blocks, lc.threads, 0, st>>>(ctl, bufs, itab, a, plog);
+    else
+      k_gather_emit<2><<<blocks, lc.threads, 0, st>>>(ctl, bufs, itab, a, plog);
   }
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }

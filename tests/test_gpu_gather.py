@@ -1,7 +1,7 @@
 """The gather-form branching pass (bucketed index, an entry writing its own row
 of the action) against the scatter form, which shares neither its index nor its
-writers, bit for bit: one entry, warps and blocks not filled, two entries a
-thread (700,001), a table at 90% load so that buckets overflow, stored zeros,
+writers, bit for bit: one entry, warps and blocks not filled, more than a
+resident grid (700,001), a table at 90% load so that buckets overflow, stored zeros,
 absent partners, controls, real, complex and Pauli matrices, both label widths."""
 
 import numpy as np
