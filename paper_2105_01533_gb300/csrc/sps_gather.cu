@@ -2221,7 +2221,7 @@ int launch_chain(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
     // one gate: the gather pass indexes only the labels with a partner and
     // reads half as much (90 us against 160 at 700,000 entries, 38 against 52
     // at 115,000); two in one layer pass: about equal (94 and 116, 206 and 163);
-    // three: 350 against 206; the eight passes of a layer of 32: 1,160 and 270
+    // three: 350 against 206; the eight passes of a layer of 32: 1,160 and 220
     if (ga.d < 3u || ga.d > kMaxAmpGates) ga.on = 0u;
   }
   a.w.words = reinterpret_cast<const uint4*>(w.words);
