@@ -735,8 +735,19 @@ long long to_q62(double x) { return std::llround(std::ldexp(x, 62)); }
 }  // namespace
 
 namespace {
-void build_bitslice_rows(const Pass& p, uint32_t nqubits, const uint64_t extra[2], bool all_out,
+bool build_bitslice_rows(const Pass& p, uint32_t nqubits, const uint64_t extra[2], bool all_out,
                          BsPass* out);
+
+// Aux rows the ops need: 3 for a counter, then one or two a phase op.
+uint32_t aux_bits_of(const std::vector<FOp>& ops) {
+  bool cnt = false;
+  uint32_t slots = 0;
+  for (const FOp& o : ops) {
+    cnt = cnt || o.a0 != 0 || o.a1 != 0;
+    if (o.ph != NO_PH) slots += o.sbit != NO_SEL ? 2u : 1u;
+  }
+  return slots + (cnt ? 3u : 0u);
+}
 }  // namespace
 
 void build_bitslice(const Pass& p, uint32_t nqubits, BsPass* out) {
@@ -794,10 +805,10 @@ bool build_bitslice_expand(const Pass& ex, const Pass& run, uint32_t nqubits, do
   }
   comb.phases.insert(comb.phases.end(), run.phases.begin(), run.phases.end());
   if (comb.phases.size() > kMaxFusedPhases + kMaxExpandGates) return false;
-  build_bitslice_rows(comb, nqubits, targets, true, out);
   // products of chunk entries keep 2^-61 of the common factor's modulus: enough
   // where every slot's factor has modulus one, not for rotations in the head
-  if (!out->direct && out->aux_bits > 0 && base > 0) return false;
+  if (base > 0 && aux_bits_of(comb.ops) > kBsDirectBits) return false;
+  if (!build_bitslice_rows(comb, nqubits, targets, true, out)) return false;
   out->expand = true;
   out->ex_d = ex.ex_d;
   out->c_re = cr;
@@ -810,14 +821,18 @@ bool build_bitslice_expand(const Pass& ex, const Pass& run, uint32_t nqubits, do
     if (r == kNoRow) return false;
     out->row_choice[r] = (int8_t)j;
   }
-  return out->aux_bits <= kMaxAuxBits && out->op_words() <= kBsMaxOps;
+  return out->op_words() <= kBsMaxOps;
 }
 
 namespace {
 
-void build_bitslice_rows(const Pass& p, uint32_t nqubits, const uint64_t extra[2], bool all_out,
+// False, with *out empty, if the ops need more than kMaxAuxBits aux rows (a run
+// alone never does: see its fire slots; with an expansion's factors it may).
+bool build_bitslice_rows(const Pass& p, uint32_t nqubits, const uint64_t extra[2], bool all_out,
                          BsPass* out) {
   *out = BsPass();
+  const uint32_t aux = aux_bits_of(p.ops);
+  if (aux > kMaxAuxBits) return false;
   BsPass& b = *out;
   b.ops.reserve(p.ops.size() + p.ops.size() / 4 + 8);
   b.nw = (nqubits + 31) / 32;
@@ -860,7 +875,6 @@ void build_bitslice_rows(const Pass& p, uint32_t nqubits, const uint64_t extra[2
   auto row_q = [&](uint32_t q) { return b.row_of[q >> 5][q & 31u]; };
   b.has_cnt = cnt;
   b.aux_row0 = row;
-  uint32_t aux = cnt ? 3u : 0u;
   std::vector<CL> factor;
   if (cnt) {
     const double r = std::sqrt(0.5);
@@ -868,8 +882,6 @@ void build_bitslice_rows(const Pass& p, uint32_t nqubits, const uint64_t extra[2
     factor.push_back(CL{0, 1});      // counter bit 1: e^{i pi/2}
     factor.push_back(CL{-1, 0});     // counter bit 2: e^{i pi}
   }
-  for (const FOp& o : p.ops)
-    if (o.ph != NO_PH) aux += o.sbit != NO_SEL ? 2u : 1u;
   b.aux_bits = aux;
   const uint8_t scratch = (uint8_t)(b.aux_row0 + aux);
   b.ones_row = scratch + 1u;
@@ -954,6 +966,7 @@ void build_bitslice_rows(const Pass& p, uint32_t nqubits, const uint64_t extra[2
   if (aux > 0) {
     b.direct = aux <= kBsDirectBits;
     b.nchunks = b.direct ? (aux > 1 ? 2u : 1u) : (aux + kBsMaxChunkBits - 1) / kBsMaxChunkBits;
+    static_assert(kMaxAuxBits <= kBsMaxChunks * kBsMaxChunkBits, "every chunk has its fields");
     uint32_t at = 0;
     for (uint32_t c = 0; c < b.nchunks; ++c) {
       const uint32_t bits = aux / b.nchunks + (c < aux % b.nchunks ? 1u : 0u);
@@ -962,6 +975,7 @@ void build_bitslice_rows(const Pass& p, uint32_t nqubits, const uint64_t extra[2
       at += bits;
     }
   }
+  return true;
 }
 
 }  // namespace

@@ -111,6 +111,7 @@ constexpr uint32_t kMaxAuxBits = 64;     // counter (3) + fire slots
 constexpr uint32_t kMaxFireSlots = kMaxAuxBits - 3;
 constexpr uint32_t kBsMaxOps = 1024;     // op words of one bit-sliced launch (kernel parameters)
 constexpr uint32_t kBsMaxChunkBits = 18; // aux bits per phase table (4 MiB)
+constexpr uint32_t kBsMaxChunks = 4;
 constexpr uint64_t kBsJitMinNnz = 1ull << 20;   // SPS_OPT_BITSLICE_JIT = 1: from this bound
 // Runs with at most this many aux bits get one table of every aux pattern's
 // phase as doubles (2^bits x 16 B, 64 MiB at most): a lookup per entry and no
@@ -144,8 +145,8 @@ struct BsPass {
   std::vector<SOp> ops;
   std::vector<long long> factors;        // aux_bits x (re, im), fixed point 2^62
   uint32_t nchunks = 0;
-  uint32_t chunk_shift[4] = {0, 0, 0, 0};
-  uint32_t chunk_bits[4] = {0, 0, 0, 0};
+  uint32_t chunk_shift[kBsMaxChunks] = {0, 0, 0, 0};
+  uint32_t chunk_bits[kBsMaxChunks] = {0, 0, 0, 0};
   // 16-byte words of the launch's op stream: one per flip or scratch AND, two
   // per general op
   uint32_t op_words() const {
@@ -292,9 +293,11 @@ constexpr uint32_t kSmallTableSlots = 8192;   // input index table, load <= 25%
 // Builds the bit-sliced form of a fused pass for an nqubits-qubit state.
 void build_bitslice(const Pass& p, uint32_t nqubits, BsPass* out);
 // The bit-sliced form of expansion pass `ex` (from |0...0>) followed by fused
-// run `run`, as one pass: false unless every expansion gate flips one qubit
-// and no output can be pruned at eps (every output factor's modulus above
-// 2 eps).
+// run `run`, as one pass: false unless every expansion gate flips one qubit,
+// no output can be pruned at eps (every output factor's modulus above 2 eps)
+// and the factors that differ with an output's choices and the run's phases
+// together need at most kMaxAuxBits aux bits (kBsDirectBits if there are any of
+// the former).
 bool build_bitslice_expand(const Pass& ex, const Pass& run, uint32_t nqubits, double eps,
                            BsPass* out);
 

@@ -1,0 +1,96 @@
+"""The host side's compiled forms, built on their own with address and
+undefined-behaviour checks: an expansion and the run after it as one bit-sliced
+pass, over phase counts around every limit of that form."""
+
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2105_01533_gb300", "csrc")
+
+EXPAND = r"""
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include "sps_internal.h"
+using namespace sps;
+static sps_gate gate(uint8_t op, uint16_t t, int c, double th) {
+  sps_gate g;
+  std::memset(&g, 0, sizeof(g));
+  g.op = op;
+  g.t0 = t;
+  if (c >= 0) g.cmask[c >> 6] = 1ull << (c & 63);
+  g.theta = th;
+  return g;
+}
+// argv: head gates, their op, controlled Rz, controlled P, T gates
+int main(int, char** v) {
+  const int head = std::atoi(v[1]), op = std::atoi(v[2]), nrz = std::atoi(v[3]), np = std::atoi(v[4]),
+            nt = std::atoi(v[5]);
+  const uint32_t nq = 60;
+  std::vector<sps_gate> g;
+  for (int q = 0; q < head; ++q) g.push_back(gate(op, q, -1, 1.2 + 0.01 * q));
+  for (int q = 0; q < head; ++q) g.push_back(gate(SPS_OP_X, 24 + q, q, 0.0));
+  for (int k = 0; k < nrz; ++k) g.push_back(gate(SPS_OP_RZ, k % head, (k + 1) % head, 0.1 + k));
+  for (int k = 0; k < np; ++k) g.push_back(gate(SPS_OP_P, k % head, (k + 1) % head, 0.1 + k));
+  for (int k = 0; k < nt; ++k) g.push_back(gate(SPS_OP_T, k % head, -1, 0.0));
+  std::vector<Pass> p;
+  KnownBits kb;
+  kb.known[0] = (1ull << nq) - 1;
+  size_t bad = 0;
+  if (compile(g.data(), g.size(), nq, 0, &p, &bad, &kb, true, true, 4, false) != SPS_OK) return 2;
+  if (p.size() < 2 || p[0].kind != PASS_EXPAND || p[1].kind != PASS_FUSED) return 3;
+  BsPass run;
+  build_bitslice(p[1], nq, &run);
+  BsPass* b = new BsPass;
+  const bool ok = build_bitslice_expand(p[0], p[1], nq, 1e-14, b);
+  uint32_t bits = 0;
+  for (uint32_t c = 0; ok && c < b->nchunks; ++c) bits += b->chunk_bits[c];
+  std::printf("%u %d %u %u %u %d\n", run.aux_bits, ok ? 1 : 0, ok ? b->aux_bits : 0u,
+              ok ? b->nchunks : 0u, bits, ok && b->direct ? 1 : 0);
+  delete b;
+  return 0;
+}
+"""
+
+
+def built(tmp, name, source):
+    cxx = shutil.which("g++")
+    if not cxx:
+        pytest.skip("needs g++")
+    src, exe = str(tmp / (name + ".cpp")), str(tmp / name)
+    with open(src, "w") as f:
+        f.write(source)
+    subprocess.run([cxx, "-std=c++17", "-O1", "-g", "-fsanitize=address,undefined",
+                    "-fno-sanitize-recover=all", "-I" + os.path.join(ROOT, "include"), "-I" + CSRC,
+                    src, os.path.join(CSRC, "sps_compile.cpp"), "-o", exe], check=True)
+    return exe
+
+
+@pytest.fixture(scope="module")
+def expand(tmp_path_factory):
+    return built(tmp_path_factory.mktemp("forms"), "expand", EXPAND)
+
+
+@pytest.mark.parametrize("head,op,nrz,np,nt", [
+    # rotations (two factors each) before the run's phases: one table of 22 bits at most
+    (5, "ry", 0, 12, 0), (5, "ry", 0, 13, 0), (4, "rx", 5, 1, 3), (4, "rx", 5, 2, 3),
+    (20, "ry", 16, 0, 0), (20, "ry", 17, 0, 0), (20, "ry", 28, 0, 0), (24, "ry", 30, 0, 1),
+    (24, "rx", 30, 1, 1),
+    # Hadamards: the run's phases alone, up to 64 bits in four tables
+    (20, "h", 11, 0, 0), (20, "h", 10, 0, 3), (20, "h", 18, 0, 0), (20, "h", 27, 0, 0),
+    (20, "h", 30, 1, 0), (20, "h", 30, 1, 1)])
+def test_expansion_and_run_within_their_tables(expand, head, op, nrz, np, nt):
+    code = {"h": 10, "rx": 11, "ry": 12}[op]
+    r = subprocess.run([expand] + [str(x) for x in (head, code, nrz, np, nt)], capture_output=True,
+                       text=True)
+    assert r.returncode == 0, r.stderr
+    run_aux, ok, aux, nchunks, bits, direct = (int(x) for x in r.stdout.split())
+    assert run_aux == 2 * nrz + np + (3 if nt else 0)
+    want = run_aux + (0 if op == "h" else 2 * head)
+    assert ok == (want <= (64 if op == "h" else 22))
+    if ok:
+        assert aux == want == bits and direct == (want <= 22) and nchunks <= 4

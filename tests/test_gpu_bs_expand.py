@@ -166,3 +166,21 @@ def test_more_phase_bits_than_one_table(n, d, cps):
     st.set_readout(None, None)
     assert abs(p - st.probability(mask, value)) < 1e-14
     st.close()
+
+
+@pytest.mark.parametrize("head,crz", [(20, 28), (20, 17), (18, 30)])
+def test_rotations_and_more_phases_than_the_form_holds(head, crz):
+    """Two factors a rotation and two a controlled Rz, up to 96 aux bits, with
+    default options: expansion and run as two launches."""
+    n = 48
+    gates = W.to_array([W.Ry(q, 1.2 + 0.01 * q) for q in range(head)] +
+                       [W.CX(q, 24 + q) for q in range(head)] +
+                       [W.CRz(k % head, (k + 1) % head, 0.1 + k) for k in range(crz)])
+    got, upd, fused = run(n, gates, 1 << 20, [(sps.SPS_OPT_BITSLICE_MIN_NNZ, 0)], True)
+    assert not fused
+    orc = OracleState(n)
+    orc.apply(gates, eps=EPS)
+    # |amplitude| <= cos(0.6)^18 = 0.04: some 50 roundings of 2^-53
+    compare_states(got, orc.get(), EPS, atol=1e-15)
+    # 1 + 2 + 4 .. before the head's gates, all outputs before the others
+    assert upd == (1 << head) - 1 + (head + crz) * (1 << head)
