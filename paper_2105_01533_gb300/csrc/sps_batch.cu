@@ -145,15 +145,15 @@ int launch_batch_reset(void* stream, BatchDesc* desc, uint32_t ncirc) {
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 
+constexpr uint32_t kBatchMaxSmemCap = 2048;
 size_t batch_smem_bytes(uint32_t smem_cap) { return (size_t)smem_cap * (64 + 16); }
 
 int batch_kernel_attr(const BatchConfig& cfg) {
-  const int smem = (int)batch_smem_bytes(cfg.smem_cap);
-  const cudaError_t e =
-      cfg.threads <= 256   ? cudaFuncSetAttribute(k_batch<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
-      : cfg.threads <= 512 ? cudaFuncSetAttribute(k_batch<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
-                           : cudaFuncSetAttribute(k_batch<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  return e == cudaSuccess ? 0 : -1;
+  const size_t smem = batch_smem_bytes(cfg.smem_cap), most = batch_smem_bytes(kBatchMaxSmemCap);
+  const bool ok = cfg.threads <= 256   ? allow_smem(k_batch<256>, smem, most)
+                  : cfg.threads <= 512 ? allow_smem(k_batch<512>, smem, most)
+                                       : allow_smem(k_batch<1024>, smem, most);
+  return ok ? 0 : -1;
 }
 
 int launch_batch(void* stream, int sms, const BatchConfig& cfg, BatchDesc* desc,
@@ -178,7 +178,7 @@ int launch_batch(void* stream, int sms, const BatchConfig& cfg, BatchDesc* desc,
 bool batch_config_ok(const BatchConfig& c) {
   if (c.threads != 256 && c.threads != 512 && c.threads != 1024) return false;
   if (c.blocks_per_sm < 1 || c.blocks_per_sm > 4) return false;
-  if (c.smem_cap != 0 && (c.smem_cap < 64 || c.smem_cap > 2048 || (c.smem_cap & (c.smem_cap - 1))))
+  if (c.smem_cap != 0 && (c.smem_cap < 64 || c.smem_cap > kBatchMaxSmemCap || (c.smem_cap & (c.smem_cap - 1))))
     return false;
   if (batch_smem_bytes(c.smem_cap) * c.blocks_per_sm > 220 * 1024) return false;
   return true;

@@ -19,6 +19,20 @@ struct __align__(16) K128a {
   uint64_t lo, hi;
 };
 
+// Lets a launch of `kern` take `smem` bytes of dynamic shared memory, of at most
+// `most`, the most any launch of it takes. The limit is the kernel's, shared by
+// every state and host thread, so it is only ever raised to `most`: set to one
+// launch's size it could be lowered by another thread before that launch.
+template <typename K>
+inline bool allow_smem(K* kern, size_t smem, size_t most) {
+  if (smem <= kDefaultSmemBytes) return true;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) ==
+      cudaSuccess)
+    return true;
+  cudaGetLastError();
+  return false;
+}
+
 // The arrays of the state `cur` names (bit 0: label buffer, bit 1: the
 // amplitudes are in the other one), without indexing the parameter struct
 // dynamically (which would copy it to local memory). pick(b, cur ^ 1) are the

@@ -2276,9 +2276,7 @@ template <int KW, bool REAL, int POST>
 static void amp_launch(int blocks, int threads, size_t smem, int sms, cudaStream_t st, Ctl* ctl,
                        Bufs bufs, const unsigned long long* itab, const AmpArgs& a,
                        unsigned long long* plog) {
-  if (POST == AMP_WALK)
-    cudaFuncSetAttribute(k_amp_layer<KW, REAL, POST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
+  allow_smem(k_amp_layer<KW, REAL, POST>, smem, kMaxOpStreamBytes);
   const int per = amp_per_sm(k_amp_layer<KW, REAL, POST>, threads, smem);
   if (per > 0 && blocks > per * sms) blocks = per * sms;
   k_amp_layer<KW, REAL, POST><<<blocks, threads, smem, st>>>(ctl, bufs, itab, a, plog);
@@ -2378,9 +2376,7 @@ int launch_gather_part(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
 template <int KW, int E, bool WALK>
 static void expand_go(int blocks, int threads, size_t smem, cudaStream_t st, Ctl* ctl, Bufs bufs,
                       const ExpandArgs& a, unsigned long long* plog) {
-  if (WALK)
-    cudaFuncSetAttribute(k_expand<KW, E, WALK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
+  allow_smem(k_expand<KW, E, WALK>, smem, kMaxOpStreamBytes);
   k_expand<KW, E, WALK><<<blocks, threads, smem, st>>>(ctl, bufs, a, plog);
 }
 

@@ -306,6 +306,11 @@ bool build_bitslice_expand(const Pass& ex, const Pass& run, uint32_t nqubits, do
 constexpr uint32_t kMaxFusedOps = 512;
 constexpr uint32_t kMaxFusedPhases = 96;
 constexpr uint32_t kDefaultMaxFusedOps = kMaxFusedOps;
+// The longest op stream: three flips or phase ops an op, each in a wide step and
+// a run of its own (the head, the run words, the steps, the step read ahead).
+constexpr uint32_t kMaxOpStreamBytes =
+    16u * (1u + (3u * kMaxFusedOps + 4u) / 4u + 4u * 3u * kMaxFusedOps + 4u);
+constexpr uint32_t kDefaultSmemBytes = 48u * 1024u;   // dynamic shared memory without asking
 
 // Validates and compiles; on a bad record returns SPS_ERR_ARG with *bad set.
 // Gate commuting queues (Sec. 3.3): rewrites the stream so that H, Rx and Ry

@@ -1288,6 +1288,7 @@ int grid_for(uint64_t work, int threads, int max_blocks) {
 // Shared memory of one block of the bit-sliced pass: 4 warps, each a tile of
 // rows x (G + 1) words.
 constexpr int kBsWarps = 4;
+constexpr size_t kBsMaxSmem = 200 * 1024;
 size_t bs_block_smem(uint32_t rows, uint32_t G) {
   return (size_t)kBsWarps * rows * (G + 1) * 4;
 }
@@ -1296,12 +1297,7 @@ size_t bs_block_smem(uint32_t rows, uint32_t G) {
 template <int KW, int NW>
 int bs_blocks_per_sm(uint32_t rows, uint32_t G) {
   const size_t smem = bs_block_smem(rows, G);
-  if (smem > 200 * 1024) return 0;
-  if (cudaFuncSetAttribute(k_fused_bs<KW, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
+  if (smem > kBsMaxSmem || !allow_smem(k_fused_bs<KW, NW>, smem, kBsMaxSmem)) return 0;
   int k = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, k_fused_bs<KW, NW>, kBsWarps * 32, smem) !=
       cudaSuccess) {
@@ -1397,7 +1393,7 @@ int fused_bs_kw(const LaunchCfg& lc, Ctl* ctl, Bufs bufs, const BsLaunch& b, uin
   const uint64_t max_blocks = (uint64_t)sms * bps;
   if (blocks > max_blocks) blocks = max_blocks;
   if (blocks < 1) blocks = 1;
-  cudaFuncSetAttribute(k_fused_bs<KW, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(k_fused_bs<KW, NW>, smem, kBsMaxSmem);
   k_fused_bs<KW, NW><<<(int)blocks, kBsWarps * 32, smem, st>>>(ctl, bufs, a, plog);
   return cudaPeekAtLastError() == cudaSuccess ? launched + 1 : -1;
 }
@@ -1458,8 +1454,7 @@ int launch_fused(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs, const 
   cudaStream_t st = (cudaStream_t)lc.stream;
   // a run of 512 dependent Y gates on 128-bit labels takes 70 KB
   auto go = [&](auto kern) {
-    if (smem > 48u * 1024u)
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(kern, smem, kMaxOpStreamBytes);
     kern<<<blocks, lc.threads, smem, st>>>(ctl, bufs, a, plog);
   };
   if (key_words == 1) {

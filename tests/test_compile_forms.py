@@ -94,3 +94,63 @@ def test_expansion_and_run_within_their_tables(expand, head, op, nrz, np, nt):
     assert ok == (want <= (64 if op == "h" else 22))
     if ok:
         assert aux == want == bits and direct == (want <= 22) and nchunks <= 4
+
+
+STREAM = r"""
+#include <cstdio>
+#include <cstring>
+#include "sps_internal.h"
+using namespace sps;
+// The longest op stream over runs of 512 ops: dependent Y gates, Y gates on all
+// qubits, Rz and Y in turn, ladders, and random gates with up to 3 controls.
+int main() {
+  unsigned long long seed = 7, longest = 0;
+  auto below = [&](unsigned n) {
+    seed = seed * 6364136223846793005ull + 1442695040888963407ull;
+    return (unsigned)((seed >> 33) % n);
+  };
+  for (uint32_t nq : {3u, 24u, 63u, 64u, 100u, 127u})
+    for (int form = 0; form < 12; ++form) {
+      std::vector<sps_gate> g;
+      for (int i = 0; i < 600; ++i) {
+        sps_gate r;
+        std::memset(&r, 0, sizeof(r));
+        auto ctl = [&](uint32_t q) { if (q != r.t0) r.cmask[q >> 6] |= 1ull << (q & 63); };
+        r.op = SPS_OP_Y;
+        r.t0 = form == 0 ? (uint16_t)(nq - 1) : (uint16_t)(i % nq);
+        r.theta = 0.3;
+        if (form == 2 && i % 20 == 1) r.op = SPS_OP_RZ;
+        if (form == 2) r.t0 = (uint16_t)(nq - 1);
+        if (form == 3) { r.op = SPS_OP_X; ctl((i + nq - 1) % nq); }
+        if (form == 4) ctl((i + nq - 1) % nq);
+        if (form > 4) {
+          const uint8_t ops[] = {SPS_OP_X, SPS_OP_Y, SPS_OP_T, SPS_OP_S, SPS_OP_Y, SPS_OP_Z};
+          r.op = ops[below(6)];
+          r.t0 = (uint16_t)below(form > 8 ? 3 : nq);
+          for (unsigned c = below(4); c; --c) ctl(below(form > 8 ? 3 : nq));
+        }
+        g.push_back(r);
+      }
+      std::vector<Pass> p;
+      size_t bad = 0;
+      if (compile(g.data(), g.size(), nq, 0, &p, &bad) != SPS_OK) return 2;
+      for (const Pass& q : p) {
+        if (q.kind != PASS_FUSED || q.ops.size() > kMaxFusedOps) return 3;
+        if (q.words.size() * sizeof(OpWord) > longest) longest = q.words.size() * sizeof(OpWord);
+      }
+    }
+  std::printf("%llu %u %u\n", longest, (unsigned)kMaxOpStreamBytes, (unsigned)kDefaultSmemBytes);
+  return 0;
+}
+"""
+
+
+def test_op_streams_within_their_limit(tmp_path):
+    """Every launch that walks an op stream asks for one limit, the longest
+    stream's; streams past the default of 48 KB do occur."""
+    out = subprocess.run([built(tmp_path, "stream", STREAM)], capture_output=True, text=True)
+    assert out.returncode == 0, out.stderr
+    longest, most, default = (int(x) for x in out.stdout.split())
+    assert default < longest <= most
+    # with the largest static shared memory of those kernels (48 KB) in an SM's 227 KB
+    assert most + default <= 227 * 1024
