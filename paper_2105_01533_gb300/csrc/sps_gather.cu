@@ -2171,22 +2171,17 @@ int launch_layer_part(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 
-// Resident blocks of k_chain per SM at `threads` (0 if the query fails).
-template <int KW, bool GRP>
-static int chain_blocks_per_sm(int threads) {
-  static int cached[5] = {-1, -1, -1, -1, -1};   // threads 32 << k, k = 0..3
-  int k = 0;
-  while (k < 4 && (32 << k) < threads) ++k;
-  if (cached[k] < 0) {
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_chain<KW, GRP>, threads, 0) !=
-        cudaSuccess) {
-      cudaGetLastError();
-      nb = 0;
-    }
-    cached[k] = nb;
-  }
-  return cached[k];
+// Resident blocks per SM of one kernel instance at `threads` and `smem` bytes of
+// dynamic shared memory (0 if the query fails).
+template <auto Kern>
+static int blocks_per_sm(int threads, size_t smem) {
+  return cached_occupancy<Kern>(threads, smem, [&] {
+    int n = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, Kern, threads, smem) == cudaSuccess)
+      return n;
+    cudaGetLastError();
+    return 0;
+  });
 }
 
 int launch_chain(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
@@ -2235,8 +2230,8 @@ int launch_chain(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
   const int sms = lc.max_blocks * lc.threads / 2048;
   const bool gr = a.grp.on != 0u;
   const int per_sm = key_words == 1
-                         ? (gr ? chain_blocks_per_sm<1, true>(threads) : chain_blocks_per_sm<1, false>(threads))
-                         : (gr ? chain_blocks_per_sm<2, true>(threads) : chain_blocks_per_sm<2, false>(threads));
+                         ? (gr ? blocks_per_sm<k_chain<1, true>>(threads, 0) : blocks_per_sm<k_chain<1, false>>(threads, 0))
+                         : (gr ? blocks_per_sm<k_chain<2, true>>(threads, 0) : blocks_per_sm<k_chain<2, false>>(threads, 0));
   if (per_sm <= 0 || sms <= 0) return 0;
   const int blocks = grid_of(nnz_bound, threads, per_sm * sms < 0x7FFF ? per_sm * sms : 0x7FFF);
   void* args[] = {&ctl, &bufs, &itab, &grp, &a, &plog};
@@ -2251,25 +2246,6 @@ int launch_chain(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
   return 1;
 }
 
-// Resident blocks per SM of one k_amp_layer instance (cached per block size
-// and dynamic shared memory; 0 if the query fails).
-template <typename K>
-static int amp_per_sm(K kern, int threads, size_t smem) {
-  static int c_threads = -1, c_per = 0;
-  static size_t c_smem = 0;
-  if (threads != c_threads || smem != c_smem) {
-    int per = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads, smem) != cudaSuccess) {
-      cudaGetLastError();
-      per = 0;
-    }
-    c_threads = threads;
-    c_smem = smem;
-    c_per = per;
-  }
-  return c_per;
-}
-
 // The attempt as one resident wave (each warp then works through many chunks,
 // so its class queues fill whole rounds).
 template <int KW, bool REAL, int POST>
@@ -2277,7 +2253,7 @@ static void amp_launch(int blocks, int threads, size_t smem, int sms, cudaStream
                        Bufs bufs, const unsigned long long* itab, const AmpArgs& a,
                        unsigned long long* plog) {
   allow_smem(k_amp_layer<KW, REAL, POST>, smem, kMaxOpStreamBytes);
-  const int per = amp_per_sm(k_amp_layer<KW, REAL, POST>, threads, smem);
+  const int per = blocks_per_sm<k_amp_layer<KW, REAL, POST>>(threads, smem);
   if (per > 0 && blocks > per * sms) blocks = per * sms;
   k_amp_layer<KW, REAL, POST><<<blocks, threads, smem, st>>>(ctl, bufs, itab, a, plog);
 }

@@ -2,6 +2,7 @@
 // of libsps. Nothing here is part of the public interface (include/sps.h).
 #pragma once
 
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 #include <string>
@@ -119,6 +120,21 @@ constexpr uint64_t kBsJitMinNnz = 1ull << 20;   // SPS_OPT_BITSLICE_JIT = 1: fro
 // expansion form the first chunk's table holds the common factor too, scaled
 // by a power of two, so an output is a fixed-point product and two conversions).
 constexpr uint32_t kBsDirectBits = 22;
+
+// The resident blocks an SM that `query` finds for a kernel instance, kept for
+// the block size and shared memory last asked for. One word holds all three, so
+// host threads may use it together; every instance has its own (instances of one
+// kernel template share a type, so the type would not tell them apart).
+template <auto Kern, typename Query>
+int cached_occupancy(int threads, size_t smem, Query query) {
+  static std::atomic<uint64_t> last{0};   // smem << 32 | threads << 16 | blocks
+  const uint64_t key = (uint64_t)smem << 32 | (uint64_t)(uint32_t)threads << 16;
+  const uint64_t v = last.load(std::memory_order_relaxed);
+  if ((v & 0xFFFFull) != 0 && (v & ~0xFFFFull) == key) return (int)(v & 0xFFFFull);
+  const int n = query();
+  if (n > 0) last.store(key | (uint64_t)(uint32_t)n, std::memory_order_relaxed);
+  return n;
+}
 
 struct BsPass {
   // the kernel compiled for this pass (sps_jit.cu), kept with the plan so a

@@ -154,3 +154,42 @@ def test_op_streams_within_their_limit(tmp_path):
     assert default < longest <= most
     # with the largest static shared memory of those kernels (48 KB) in an SM's 227 KB
     assert most + default <= 227 * 1024
+
+
+OCCUPANCY = r"""
+#include <cstdio>
+#include <thread>
+#include "sps_internal.h"
+using namespace sps;
+static int kernel_a() { return 5; }
+static int kernel_b() { return 3; }
+template <int (*K)()>
+static int ask(int threads, size_t smem, int* queries) {
+  return cached_occupancy<K>(threads, smem, [&] { ++*queries; return smem > 100000 ? 0 : K() + threads / 128; });
+}
+int main() {
+  int q = 0;
+  if (ask<kernel_a>(128, 64, &q) != 6 || ask<kernel_b>(128, 64, &q) != 4) return 2;
+  if (ask<kernel_a>(128, 64, &q) != 6 || q != 2) return 3;          // kept, each its own
+  if (ask<kernel_a>(256, 64, &q) != 7 || ask<kernel_a>(256, 80, &q) != 7 || q != 4) return 4;
+  if (ask<kernel_a>(256, 200000, &q) != 0 || ask<kernel_a>(256, 200000, &q) != 0 || q != 6) return 5;
+  bool bad[2] = {false, false};
+  auto work = [&](int t) {
+    int n = 0;
+    for (int i = 0; i < 200000; ++i) {
+      const int threads = (i + t) & 1 ? 128 : 256;
+      if (ask<kernel_b>(threads, 16 * (size_t)t, &n) != 3 + threads / 128) bad[t] = true;
+    }
+  };
+  std::thread other(work, 1);
+  work(0);
+  other.join();
+  return bad[0] || bad[1] ? 6 : 0;
+}
+"""
+
+
+def test_occupancy_kept_per_kernel_instance(tmp_path):
+    """Instances of one type, other block sizes and shared memory, failures, and
+    two threads: an answer is never another question's."""
+    assert subprocess.run([built(tmp_path, "occupancy", OCCUPANCY)]).returncode == 0
