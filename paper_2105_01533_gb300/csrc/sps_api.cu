@@ -667,16 +667,26 @@ static uint64_t bound_after(const Pass& p, uint64_t b, uint64_t capacity) {
   return b < capacity ? b : capacity;
 }
 
-// A fresh 16-bit epoch for the index table; when it wraps, every slot is made
-// free again (which also drops the label index of amplitude-only passes).
-static sps_status next_epoch(sps_state* s, const LaunchCfg& lc) {
-  if (++s->epoch == 0x10000u) {
+// Fresh 16-bit epochs for the index table, first .. first + count - 1; when they
+// wrap, every slot is made free again (which also drops the label index of
+// amplitude-only passes). A launch that takes several draws them at once: the
+// clear runs before the launch, so slots it wrote with epochs from before a wrap
+// among them would stay and count as current one turn of the counter later.
+static sps_status next_epochs(sps_state* s, const LaunchCfg& lc, uint32_t count, uint32_t* first) {
+  if (s->epoch + count >= 0x10000u) {
     if (launch_itab_clear(lc, s->itab, 1ull << s->itab_log2) < 0) return cuda_ok(cudaGetLastError());
     s->counters.kernel_launches += 1;
-    s->epoch = 1;
+    s->epoch = 0;
     s->amp_force = true;
   }
+  *first = s->epoch + 1;
+  s->epoch += count;
   return SPS_OK;
+}
+
+static sps_status next_epoch(sps_state* s, const LaunchCfg& lc) {
+  uint32_t first;
+  return next_epochs(s, lc, 1, &first);
 }
 
 // The amplitude-only attempt of a run of gather-form branching passes, d gates
@@ -806,25 +816,20 @@ static bool launch_fallback_chain(sps_state* s, const LaunchCfg& lc, const Apply
   ChainStepDesc steps[kChainSteps];
   uint32_t nsteps = 0;
   const uint32_t first_serial = s->pass_serial + 1;
-  const sps_status ge = next_epoch(s, lc);   // the group stage's index
+  uint32_t grp_epoch;   // the group stage's index; the steps' follow
+  const sps_status ge = next_epochs(s, lc, 1u + (uint32_t)(amp_end - pi), &grp_epoch);
   if (ge != SPS_OK) {
     *err = ge;
     return true;
   }
-  const uint32_t grp_epoch = s->epoch;
   for (size_t k = pi; k < amp_end; ++k) {
     const Pass& q = passes[k];
     ChainStepDesc& d = steps[nsteps++];
     std::memset(&d, 0, sizeof(d));
     const uint32_t serial = ++s->pass_serial;
     const uint64_t tag = ((uint64_t)s->apply_serial << 32) | (q.first_gate & 0xFFFFFFFFull);
-    const sps_status es = next_epoch(s, lc);   // a wrap clears the table before the launch
-    if (es != SPS_OK) {
-      *err = es;
-      return true;
-    }
     d.kind = q.kind;
-    d.epoch = s->epoch;
+    d.epoch = grp_epoch + nsteps;
     if (q.kind == PASS_LAYER) {
       LayerLaunch& l = d.lay;
       l.fallback = 1;

@@ -129,3 +129,44 @@ def test_sector_fills_as_its_passes_fill_it():
     for p in parts:
         orc.apply(p, eps=1e-14)
     compare_states(got, orc.get(), 1e-14)
+
+
+def test_epochs_of_one_launch_do_not_wrap():
+    """The fallback launch draws an epoch for its group stage and one a pass. Drawn
+    across the wrap of the 16-bit counter, one turn later the slots it left would
+    pass for labels of a state that lies over the older one's entries (2,048
+    labels, of which the later states hold 1,025 and lack the others)."""
+    n, nq = 2048, 20
+    lo = np.arange(n, dtype=np.uint64)
+    rng = np.random.default_rng(3)
+    re, im = rng.normal(size=n), rng.normal(size=n)
+    st = sps.SparseState(nq, 8 * n)
+    for o, v in ((sps.SPS_OPT_SMALL_RUN_CAP, 0), (sps.SPS_OPT_EXPAND, 0),
+                 (sps.SPS_OPT_LAYER_GATES, 1), (sps.SPS_OPT_AMP_ONLY, 0)):
+        st.set_option(o, v)
+    one = [np.zeros(1, np.uint64), np.zeros(1, np.uint64), np.ones(1), np.zeros(1)]
+
+    def passes(count):   # one epoch each
+        st.set_amplitudes(*one)
+        st.apply(np.tile(W.to_array([W.H(19)]), count), 1e-14)
+
+    passes(65532)
+    st.set_option(sps.SPS_OPT_AMP_ONLY, 1)
+    st.set_amplitudes(np.zeros_like(lo), lo, re, im)
+    st.apply(W.to_array([W.H(12), W.H(13), W.H(14)]), 1e-14)   # epochs 65533 ..
+    assert st.nnz() == 8 * n
+    st.set_option(sps.SPS_OPT_AMP_ONLY, 0)
+    passes(65521)
+    m = n // 2 + 1
+    a = np.zeros(n, np.complex128)
+    a[:m] = re[:m] + 1j * im[:m]
+    r = np.sqrt(0.5)
+    want = np.concatenate([r * a[:n // 2] + r * a[n // 2:], r * a[:n // 2] - r * a[n // 2:]])
+    for _ in range(14):   # up to and past the next wrap
+        st.set_amplitudes(np.zeros_like(lo[:m]), lo[:m], re[:m], im[:m])
+        st.apply(W.to_array([W.H(10)]), 1e-14)
+        _, klo, kre, kim = st.get_amplitudes()
+        np.testing.assert_array_equal(klo, lo)
+        # two products and a sum
+        np.testing.assert_allclose(kre + 1j * kim, want, rtol=0, atol=2e-15)
+    st.close()
