@@ -255,14 +255,18 @@ void sps::hook_free(void* p, size_t bytes, void* stream) {
 
 double* sps::device_view(const void* p, int device, bool host_too) {
   cudaPointerAttributes at;
-  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+  int current = -1;
+  if (cudaGetDevice(&current) != cudaSuccess || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();
     return nullptr;
   }
-  const bool ok = (at.type == cudaMemoryTypeDevice && at.device == device) ||
-                  (host_too && at.type == cudaMemoryTypeHost);
-  if (!ok || (reinterpret_cast<uintptr_t>(at.devicePointer) & 7u)) return nullptr;
-  return static_cast<double*>(at.devicePointer);
+  const MemKind kind = at.type == cudaMemoryTypeDevice ? MEM_DEVICE
+                       : at.type == cudaMemoryTypeHost ? MEM_PINNED
+                                                       : MEM_OTHER;
+  return kernel_may_write(kind, at.device, device, current,
+                          reinterpret_cast<uintptr_t>(at.devicePointer), host_too)
+             ? static_cast<double*>(at.devicePointer)
+             : nullptr;
 }
 
 namespace {

@@ -636,8 +636,17 @@ int launch_copy_entries(void* stream, SoA s, uint64_t n, uint64_t* hi, uint64_t*
 int launch_zphase(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs, const uint64_t z[2],
                   const uint64_t c[2], double cs, double sn, uint32_t ngates, uint64_t nnz_bound,
                   unsigned long long* plog);
-// The address a kernel on `device` may write `words` doubles of the caller's at:
-// device memory of that device or pinned host memory, 8-byte aligned; else null.
+// Whether a kernel of a state on `device` may write words at `address`, a device
+// address of memory of this kind and owner: memory of that device or (host_too)
+// pinned host memory, 8-byte aligned, while that device is the current one: a
+// kernel is launched on the current device, a copy on its stream's.
+enum MemKind { MEM_DEVICE, MEM_PINNED, MEM_OTHER };
+inline bool kernel_may_write(MemKind kind, int owner, int device, int current, uintptr_t address,
+                             bool host_too) {
+  if (current != device || address == 0 || (address & 7u)) return false;
+  return kind == MEM_DEVICE ? owner == device : kind == MEM_PINNED && host_too;
+}
+// The address at which a kernel may write the caller's words at p, or null.
 double* device_view(const void* p, int device, bool host_too);
 int launch_probability(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
                        uint64_t mask_lo, uint64_t mask_hi, uint64_t val_lo, uint64_t val_hi,

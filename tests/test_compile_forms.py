@@ -193,3 +193,31 @@ def test_occupancy_kept_per_kernel_instance(tmp_path):
     """Instances of one type, other block sizes and shared memory, failures, and
     two threads: an answer is never another question's."""
     assert subprocess.run([built(tmp_path, "occupancy", OCCUPANCY)]).returncode == 0
+
+
+WRITES = r"""
+#include "sps_internal.h"
+using namespace sps;
+int main() {
+  const uintptr_t a = 0x7f0000001000;
+  struct { MemKind kind; int owner, device, current; uintptr_t at; bool host_too, want; } t[] = {
+      {MEM_DEVICE, 0, 0, 0, a, false, true},  {MEM_DEVICE, 0, 0, 0, a + 8, true, true},
+      {MEM_DEVICE, 1, 1, 1, a, false, true},  {MEM_PINNED, 0, 0, 0, a, true, true},
+      {MEM_PINNED, 1, 0, 0, a, true, true},                       // pinned for every device
+      {MEM_DEVICE, 0, 0, 1, a, false, false},                     // another device is current
+      {MEM_PINNED, 0, 0, 1, a, true, false},  {MEM_DEVICE, 1, 0, 0, a, false, false},
+      {MEM_DEVICE, 1, 0, 1, a, false, false}, {MEM_PINNED, 0, 0, 0, a, false, false},
+      {MEM_OTHER, 0, 0, 0, a, true, false},   {MEM_DEVICE, 0, 0, 0, a + 4, false, false},
+      {MEM_DEVICE, 0, 0, 0, 0, false, false}, {MEM_DEVICE, 0, 0, -1, a, false, false},
+  };
+  for (const auto& c : t)
+    if (kernel_may_write(c.kind, c.owner, c.device, c.current, c.at, c.host_too) != c.want) return 1;
+  return 0;
+}
+"""
+
+
+def test_who_writes_the_callers_memory(tmp_path):
+    """A read-back or readout goes by kernel only where a kernel can be launched and
+    can write: else by copies, as with another device current."""
+    assert subprocess.run([built(tmp_path, "writes", WRITES)]).returncode == 0
