@@ -191,6 +191,22 @@ __device__ __forceinline__ void add_if(uint32_t miss, const uint4& t, uint64_t& 
       : "l"(a), "r"(miss));
 }
 
+template <bool WIDE>
+__device__ __forceinline__ void apply_if(uint32_t miss, const uint4& t, uint32_t& w0, uint32_t& w1,
+                                         uint32_t& w2, uint32_t& w3, uint64_t a, uint64_t& ph) {
+  if (WIDE)
+    asm("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %10, 0;\n\t@p xor.b32 %0, %0, %5;\n\t"
+        "@p xor.b32 %1, %1, %6;\n\t@p xor.b32 %2, %2, %7;\n\t@p xor.b32 %3, %3, %8;\n\t"
+        "@p add.u64 %4, %4, %9;\n\t}"
+        : "+r"(w0), "+r"(w1), "+r"(w2), "+r"(w3), "+l"(ph)
+        : "r"(t.x), "r"(t.y), "r"(t.z), "r"(t.w), "l"(a), "r"(miss));
+  else
+    asm("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %6, 0;\n\t@p xor.b32 %0, %0, %3;\n\t"
+        "@p xor.b32 %1, %1, %4;\n\t@p add.u64 %2, %2, %5;\n\t}"
+        : "+r"(w0), "+r"(w1), "+l"(ph)
+        : "r"(t.x), "r"(t.y), "l"(a), "r"(miss));
+}
+
 // One step of the op stream on E labels: the conditions of both ops are
 // evaluated on the labels as they are before the step (the ops of a level do
 // not read what the others flip), then FLIP: the targets of those that hold
@@ -222,8 +238,33 @@ __device__ __forceinline__ void walk_step(const uint4 (&o)[WIDE ? 4 : 2], uint32
   }
 }
 
-// The runs of an op stream from run r on as long as they have this width (see
-// OpWord's comment for the layout); q: the first step. The next step's words
+// A run of single steps (ANY: of either kind, see OpWord), in order. The loads of
+// an unrolled group go out together.
+template <bool WIDE, bool ANY, int E>
+__device__ __forceinline__ void walk_singles(uint32_t steps, const uint4* __restrict__& q,
+                                             uint32_t (&w0)[E], uint32_t (&w1)[E],
+                                             uint32_t (&w2)[E], uint32_t (&w3)[E],
+                                             uint64_t (&ph)[E]) {
+  constexpr uint32_t S = (WIDE ? 2u : 1u) + (ANY ? 1u : 0u);   // words a step
+  constexpr int U = WIDE || ANY ? 4 : 8;
+#pragma unroll U
+  for (uint32_t k = 0; k < steps; ++k) {
+    const uint4 c = q[S * k];
+    const uint4 t = WIDE ? q[S * k + 1] : make_uint4(c.z, c.w, 0u, 0u);
+    const uint2 a = ANY ? *reinterpret_cast<const uint2*>(q + S * k + S - 1) : make_uint2(0u, 0u);
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      uint32_t miss = ((w0[e] & c.x) ^ c.x) | ((w1[e] & c.y) ^ c.y);
+      if (WIDE) miss |= ((w2[e] & c.z) ^ c.z) | ((w3[e] & c.w) ^ c.w);
+      if (ANY) apply_if<WIDE>(miss, t, w0[e], w1[e], w2[e], w3[e], ((uint64_t)a.y << 32) | a.x, ph[e]);
+      else flip_if<WIDE>(miss, t, w0[e], w1[e], w2[e], w3[e]);
+    }
+  }
+  q += S * steps;
+}
+
+// The runs of pairs of an op stream from run r on as long as they have this width
+// (see OpWord's comment for the layout); q: the first step. The next step's words
 // are loaded before the current one is worked, so a step costs its own latency
 // and not a load's.
 template <bool WIDE, int E>
@@ -238,7 +279,7 @@ __device__ __forceinline__ void walk_runs(const uint32_t* __restrict__ runs, uin
   for (int i = 0; i < S; ++i) cur[i] = q[i];
   uint32_t run = runs[r];
   do {
-    const uint32_t nf = run & 0xFFFFu, np = (run >> 16) & 0x7FFFu;
+    const uint32_t nf = run & 0xFFFFu, np = (run >> 16) & 0x1FFFu;
     run = runs[++r];
 #pragma unroll 2
     for (uint32_t k = 0; k < nf; ++k) {
@@ -258,7 +299,7 @@ __device__ __forceinline__ void walk_runs(const uint32_t* __restrict__ runs, uin
 #pragma unroll
       for (int i = 0; i < S; ++i) cur[i] = nxt[i];
     }
-  } while (r < nruns && ((run & kRunWide) != 0u) == WIDE);
+  } while (r < nruns && (run & (kRunWide | kRunSingle)) == (WIDE ? kRunWide : 0u));
 }
 
 // Runs a fused pass's encoded op stream (in shared or global memory; every
@@ -285,10 +326,21 @@ __device__ __forceinline__ void walk_ops_n(const uint4* __restrict__ sq, uint32_
   const uint32_t* __restrict__ runs = reinterpret_cast<const uint32_t*>(sq + 1);
   const uint4* __restrict__ q = sq + head.y;
   for (uint32_t r = 0; r < head.x;) {
-    if (KW == 2 && (runs[r] & kRunWide) != 0u)
-      walk_runs<true, E>(runs, head.x, r, q, w0, w1, w2, w3, ph);
-    else
-      walk_runs<false, E>(runs, head.x, r, q, w0, w1, w2, w3, ph);
+    const uint32_t run = runs[r], steps = run & 0xFFFFu;
+    const bool wide = KW == 2 && (run & kRunWide) != 0u;
+    if ((run & kRunSingle) == 0u) {
+      if (wide) walk_runs<true, E>(runs, head.x, r, q, w0, w1, w2, w3, ph);
+      else walk_runs<false, E>(runs, head.x, r, q, w0, w1, w2, w3, ph);
+      continue;
+    }
+    ++r;
+    if ((run & kRunAny) == 0u) {
+      if (wide) walk_singles<true, false, E>(steps, q, w0, w1, w2, w3, ph);
+      else walk_singles<false, false, E>(steps, q, w0, w1, w2, w3, ph);
+    } else {
+      if (wide) walk_singles<true, true, E>(steps, q, w0, w1, w2, w3, ph);
+      else walk_singles<false, true, E>(steps, q, w0, w1, w2, w3, ph);
+    }
   }
 #pragma unroll
   for (int e = 0; e < E; ++e) {

@@ -209,12 +209,16 @@ struct BsPass {
 // conditions of a pair are evaluated together; phase ops wait for a level that
 // one of them cannot outwait and go out there, in pairs too.
 //   word 0            {runs, words before the first step, 0, 0}
-//   then              a 32-bit word per run: flip pairs | phase pairs << 16 |
+//   then              a 32-bit word per run: steps | phase pairs << 16 |
 //                     kRunWide if one of its ops reads or flips qubits 64..127
+//                     | kRunSingle, kRunAny: its form
 //   then              the steps: two ops of one word {c, t} (32-bit halves of
 //                     qubits 0..63), or, in a wide run, of two words, c then t
 //                     (128 bits; a phase op's word in its low half); a wide
 //                     step of zeros at the end (read ahead).
+// A run's form: pairs of flips, then pairs of phase ops; kRunSingle: single flips;
+// kRunSingle | kRunAny: single ops of either kind, the words of a flip (zeros
+// in a phase op) and then one of the phase (zeros in a flip).
 // Short stretches of narrow levels between wide ones are made wide too (a
 // change of width refills the read-ahead).
 // Why pairs: with few labels a thread's time is the latency of the chain
@@ -223,9 +227,12 @@ struct BsPass {
 // of one form with a header each (three to four ops long in random circuits),
 // and a header cost a load, a branch and a refilled pipeline. 512 ops on 4,096
 // 64-bit labels: 42 us before, 18 now; on 65,536 128-bit labels 70 and 26.
+// Why singles: see encode_ops.
 struct OpWord { uint32_t x, y, z, w; };
 static_assert(sizeof(OpWord) == 16, "OpWord layout");
 constexpr uint32_t kRunWide = 1u << 31;
+constexpr uint32_t kRunSingle = 1u << 30;
+constexpr uint32_t kRunAny = 1u << 29;
 constexpr uint32_t kOpCountShift = 61;   // phase word: counter above the fire slots
 struct Pass;
 // Encodes the pass's ops (p.words) and builds its fire-slot tables (p.ftab).

@@ -221,3 +221,194 @@ def test_who_writes_the_callers_memory(tmp_path):
     """A read-back or readout goes by kernel only where a kernel can be launched and
     can write: else by copies, as with another device current."""
     assert subprocess.run([built(tmp_path, "writes", WRITES)]).returncode == 0
+
+
+WALK = r"""
+#include <cstdio>
+#include <cstring>
+#include "sps_internal.h"
+using namespace sps;
+typedef unsigned long long u64;
+static u64 seed = 11;
+static u64 rnd() {
+  seed = seed * 6364136223846793005ull + 1442695040888963407ull;
+  u64 x = seed;
+  x ^= x >> 31;
+  return x * 0x9E3779B97F4A7C15ull;
+}
+static unsigned below(unsigned n) { return (unsigned)((rnd() >> 33) % n); }
+struct Label { u64 k[2]; unsigned cnt; u64 fire; };
+// the ops in order: pi/4 steps and the slots of the phases that apply, as met
+static void direct(const Pass& p, Label& l) {
+  unsigned slot = 0;
+  for (const FOp& o : p.ops) {
+    const unsigned s0 = slot, s1 = slot + 1;
+    if (o.ph != NO_PH) slot += o.sbit != NO_SEL ? 2 : 1;
+    if ((l.k[0] & o.c[0]) != o.c[0] || (l.k[1] & o.c[1]) != o.c[1]) continue;
+    const bool sel = o.sbit != NO_SEL && ((l.k[o.sbit >> 6] >> (o.sbit & 63)) & 1ull);
+    l.cnt += sel ? o.a1 : o.a0;
+    if (o.ph != NO_PH) l.fire |= 1ull << (sel ? s1 : s0);
+    l.k[0] ^= o.t[0];
+    l.k[1] ^= o.t[1];
+  }
+  l.cnt &= 7u;
+}
+static u64 forms[6];
+static void stream(const Pass& p, Label& l) {
+  if (p.words.empty()) return;
+  const OpWord* W = p.words.data();
+  const uint32_t* runs = &W[1].x;
+  size_t q = W[0].y;
+  u64 ph = 0;
+  auto holds = [&](u64 c0, u64 c1) { return (l.k[0] & c0) == c0 && (l.k[1] & c1) == c1; };
+  auto two = [](uint32_t a, uint32_t b) { return (u64)b << 32 | a; };
+  for (uint32_t r = 0; r < W[0].x; ++r) {
+    const uint32_t run = runs[r], n = run & 0xFFFFu, np = (run >> 16) & 0x1FFFu;
+    const bool wide = run & kRunWide, any = run & kRunAny;
+    const int S = wide ? 2 : 1;
+    forms[(wide ? 3 : 0) + (run & kRunSingle ? (any ? 2 : 1) : 0)] += 1;
+    if (run & kRunSingle) {
+      for (uint32_t k = 0; k < n; ++k, q += S + (any ? 1 : 0)) {
+        if (!holds(two(W[q].x, W[q].y), wide ? two(W[q].z, W[q].w) : 0)) continue;
+        const OpWord t = wide ? W[q + 1] : OpWord{W[q].z, W[q].w, 0, 0};
+        l.k[0] ^= two(t.x, t.y);
+        l.k[1] ^= two(t.z, t.w);
+        if (any) ph += two(W[q + S].x, W[q + S].y);
+      }
+      continue;
+    }
+    for (uint32_t k = 0; k < n + np; ++k) {   // both conditions on the label before the step
+      bool on[2];
+      OpWord t[2];
+      for (int h = 0; h < 2; ++h, q += S) {
+        on[h] = holds(two(W[q].x, W[q].y), wide ? two(W[q].z, W[q].w) : 0);
+        t[h] = wide ? W[q + 1] : OpWord{W[q].z, W[q].w, 0, 0};
+      }
+      for (int h = 0; h < 2; ++h)
+        if (on[h]) {
+          if (k < n) {
+            l.k[0] ^= two(t[h].x, t[h].y);
+            l.k[1] ^= two(t[h].z, t[h].w);
+          } else {
+            ph += two(t[h].x, t[h].y);
+          }
+        }
+    }
+  }
+  if (q + 4 != p.words.size()) std::printf("length %zu of %zu\n", q, p.words.size());
+  l.cnt = (unsigned)(ph >> kOpCountShift) & 7u;
+  l.fire = ph & ((1ull << kOpCountShift) - 1);
+}
+int main() {
+  int bad = 0;
+  for (uint32_t nq : {2u, 5u, 24u, 63u, 64u, 70u, 127u})
+    for (int round = 0; round < 220; ++round) {
+      const int form = round % 11;
+      std::vector<sps_gate> g;
+      const int count = round % 3 == 0 ? 1 + (int)below(12) : 20 + (int)below(500);
+      for (int i = 0; i < count; ++i) {
+        sps_gate r;
+        std::memset(&r, 0, sizeof(r));
+        auto ctl = [&](uint32_t q) { if (q != r.t0) r.cmask[q >> 6] |= 1ull << (q & 63); };
+        r.op = SPS_OP_X;
+        r.t0 = (uint16_t)(i % nq);
+        r.theta = 0.1 + i;
+        const uint8_t all[] = {SPS_OP_X, SPS_OP_Y, SPS_OP_Z, SPS_OP_S, SPS_OP_TDG, SPS_OP_P, SPS_OP_RZ};
+        if (form == 3) r.t0 = (uint16_t)below(3 < nq ? 3 : nq);
+        if (form == 6) r.t0 = (uint16_t)below(nq);
+        if (form > 6) r.t0 = (uint16_t)(form == 10 ? nq - 1 - below(2) : below(nq));
+        if (form < 4) ctl((i + nq - 1) % nq);                           // ladders
+        if (form == 1 && i % 3 == 1) r.op = SPS_OP_T;                  // with phases between
+        if (form == 2 && i % 40 > 20) r.op = all[below(7)];
+        if (form == 4) r.op = SPS_OP_Y, r.t0 = (uint16_t)(nq - 1);
+        if (form == 5) { r.op = SPS_OP_Y; ctl(below(nq)); }
+        if (form == 6) { ctl(below(nq)); ctl(below(nq)); }
+        if (form > 6) {
+          r.op = all[below(7)];
+          for (unsigned c = below(form == 9 ? 7 : 3); c; --c) ctl(below(nq));
+        }
+        g.push_back(r);
+      }
+      std::vector<Pass> ps;
+      size_t at = 0;
+      KnownBits kb;
+      if (round & 1) { kb.known[0] = rnd() & rnd(); kb.known[0] &= nq < 64 ? (1ull << nq) - 1 : ~0ull; }
+      const KnownBits k0 = kb;
+      if (compile(g.data(), g.size(), nq, 0, &ps, &at, round & 1 ? &kb : nullptr, false, true) != SPS_OK)
+        return 2;
+      for (int e = 0; e < 40; ++e) {
+        Label l{{rnd(), rnd()}, 0, 0};
+        l.k[0] &= nq < 64 ? (1ull << nq) - 1 : ~0ull;
+        l.k[1] &= nq > 64 ? (1ull << (nq - 64)) - 1 : 0ull;
+        l.k[0] &= ~k0.known[0];   // (known to be 0)
+        for (const Pass& p : ps) {
+          Label a = l, b = l;
+          a.cnt = b.cnt = 0;
+          a.fire = b.fire = 0;
+          direct(p, a);
+          stream(p, b);
+          if (a.k[0] != b.k[0] || a.k[1] != b.k[1] || a.cnt != b.cnt || a.fire != b.fire) ++bad;
+          l = a;
+        }
+      }
+    }
+  std::printf("%d %llu %llu %llu %llu %llu %llu\n", bad, forms[0], forms[1], forms[2], forms[3], forms[4], forms[5]);
+  return bad != 0;
+}
+"""
+
+
+def test_op_streams_do_what_their_ops_do(tmp_path):
+    """Every form of run, on labels of both widths, with and without known qubits:
+    the stream's flips, pi/4 steps and phase slots against the ops one by one."""
+    out = subprocess.run([built(tmp_path, "walk", WALK)], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout + out.stderr
+    words = [int(x) for x in out.stdout.split()]
+    assert words[0] == 0 and min(words[1:]) > 0, words
+
+
+LENGTHS = r"""
+#include <cstdio>
+#include <cstring>
+#include "sps_internal.h"
+using namespace sps;
+// words and pairs of flips of the streams of: a CNOT ladder, Y gates on one qubit,
+// CNOTs on 24 disjoint pairs
+int main() {
+  for (int form = 0; form < 3; ++form) {
+    std::vector<sps_gate> g;
+    auto cx = [&](int a, int b, int t) {
+      sps_gate r;
+      std::memset(&r, 0, sizeof(r));
+      r.op = SPS_OP_X;
+      r.t0 = (uint16_t)t;
+      r.cmask[0] = (a >= 0 ? 1ull << a : 0ull) | (b >= 0 ? 1ull << b : 0ull);
+      g.push_back(r);
+    };
+    for (int i = 0; form == 0 && i < 480; ++i) cx(i % 48, -1, (i + 1) % 48);
+    for (int i = 0; form == 1 && i < 480; ++i) {
+      cx(-1, -1, 3);
+      g.back().op = SPS_OP_Y;
+    }
+    for (int i = 0; form == 2 && i < 480; ++i) cx(2 * (i % 24), -1, 2 * (i % 24) + 1);
+    std::vector<Pass> p;
+    size_t bad = 0;
+    if (compile(g.data(), g.size(), 50, 0, &p, &bad) != SPS_OK || p.size() != 1) return 2;
+    uint32_t pairs = 0;
+    for (uint32_t r = 0; r < p[0].words[0].x; ++r)
+      pairs += (&p[0].words[1].x)[r] & kRunSingle ? 0u : (&p[0].words[1].x)[r] & 0xFFFFu;
+    std::printf("%zu %u\n", p[0].words.size() - p[0].words[0].y - 4, pairs);
+  }
+  return 0;
+}
+"""
+
+
+def test_no_half_empty_pairs_on_serial_chains(tmp_path):
+    """A chain of flips that each read what the last one flipped is single steps, a
+    word a flip (as pairs it would be two); flips that wait for nothing are pairs."""
+    out = subprocess.run([built(tmp_path, "lengths", LENGTHS)], capture_output=True, text=True)
+    assert out.returncode == 0, out.stderr
+    ladder, ys, disjoint = ([int(x) for x in line.split()] for line in out.stdout.splitlines())
+    assert ladder == [480, 0] and disjoint == [480, 240]
+    assert ys[1] <= 1   # beside the phase ops that read nothing

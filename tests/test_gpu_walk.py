@@ -91,3 +91,44 @@ def test_walk_in_one_block_and_after_expansion(make):
         orc.apply(g, eps=EPS)
         compare_states(st.get_amplitudes(), orc.get(), EPS)
         st.close()
+
+
+def ladder(nq):
+    """Every gate reads what the last one flipped: single flips."""
+    return [W.CX(i % nq, (i + 1) % nq) for i in range(300)]
+
+
+def adder(nq):
+    """One and two flips a level in turn."""
+    n = (nq - 1) // 2
+    up = [(2 * n if i == 0 else i - 1, i, n + i) for i in range(n)]
+    return [g for c, x, y in up for g in (W.CX(x, y), W.CX(x, c), W.CCX(c, y, x))] + \
+           [g for c, x, y in up[::-1] for g in (W.CCX(c, y, x), W.CX(x, c), W.CX(c, y))]
+
+
+def ladder_with_phases(nq):
+    """A phase op between the flips it waits for: steps of either kind, a long
+    stretch of flips alone, then a level with many phase ops."""
+    out = []
+    for i in range(20):
+        a, b = i % nq, (i + 1) % nq
+        out += [W.CX(a, b), W.Rz(b, 0.1 + i), W.CX(a, b), W.Y(b, a)]
+    return out + ladder(nq) + [W.CZ(i % nq, (i + 3) % nq) for i in range(40)] + [W.CX(0, 1), W.S(1)]
+
+
+@pytest.mark.parametrize("small", [0, 2048])
+@pytest.mark.parametrize("nq,log2n", [(9, 5), (24, 0), (63, 10), (64, 7), (100, 11), (127, 12)])
+@pytest.mark.parametrize("make", [ladder, adder, ladder_with_phases])
+def test_single_steps(make, nq, log2n, small):
+    g = W.to_array([W.H(q) for q in range(log2n)] + make(nq))
+    for walk in (0, 1):
+        st = sps.SparseState(nq, 1 << log2n)
+        st.set_option(sps.SPS_OPT_SMALL_RUN_CAP, small)
+        st.set_option(sps.SPS_OPT_BITSLICE_MIN_OPS, 0)
+        st.set_option(sps.SPS_OPT_EXPAND_WALK, walk)
+        st.set_option(sps.SPS_OPT_FOLD, 0)
+        st.apply(g, EPS)
+        orc = OracleState(nq)
+        orc.apply(g, eps=EPS)
+        compare_states(st.get_amplitudes(), orc.get(), EPS)
+        st.close()
