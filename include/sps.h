@@ -448,7 +448,8 @@ sps_status sps_get_counters(sps_state* s, sps_counters* out);
  * launch also applied the phase/permutation run after the branching gates,
  * bit 3 (kind 1) bit-sliced form, bit 4 (kind 1) the form compiled for this
  * run (SPS_OPT_BITSLICE_JIT), bit 5 (kind 7) the launch also summed the
- * registered readout (sps_set_readout). label_bytes: 8 or 16. */
+ * registered readout (sps_set_readout), bit 6 (kind 11) the run was taken as
+ * groups, bit 7 (kind 11) that was tried. label_bytes: 8 or 16. */
 typedef struct sps_kernel_record {
   uint32_t kind;
   uint32_t pass_serial;

@@ -637,8 +637,9 @@ sps_status sps_profile_read(sps_state* s, sps_kernel_record* out, size_t cap, si
     out[i].ms = ms;
     out[i].nops = p.nops;
     out[i].n_in = s->hlog[2 * i];
-    out[i].n_out = s->hlog[2 * i + 1];
-    out[i].flags = p.flags;
+    const unsigned long long last = s->hlog[2 * i + 1];
+    out[i].n_out = last & ~(kLogGroupsTried | kLogGroupsTook);
+    out[i].flags = p.flags | (last & kLogGroupsTook ? 64u : 0u) | (last & kLogGroupsTried ? 128u : 0u);
     out[i].label_bytes = 8u * (uint32_t)s->kw;
     s->event_pool.push_back(p.start);
     s->event_pool.push_back(p.stop);

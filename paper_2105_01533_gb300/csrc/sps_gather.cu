@@ -2081,7 +2081,8 @@ __global__ void __launch_bounds__(256) k_chain(Ctl* ctl, Bufs bufs, unsigned lon
     chain_walk<KW>(ctl, bufs, a.w);
     grid_barrier(ctl, serial + 1u, tag);
   }
-  if (plog && blockIdx.x == 0 && threadIdx.x == 0) plog[1] = ctl->nnz;
+  if (plog && blockIdx.x == 0 && threadIdx.x == 0)
+    plog[1] = ctl->nnz | (GRP ? kLogGroupsTried : 0ull) | (grouped ? kLogGroupsTook : 0ull);
 }
 
 // The barrier's bounded wait, exercised: `rounds` barriers over the grid; block

@@ -397,6 +397,10 @@ struct Ctl {
   unsigned long long chunk_next;
 };
 
+// Beside the entry count a profiled fallback launch writes last: the group stage
+// was tried; it produced the state.
+constexpr unsigned long long kLogGroupsTried = 1ull << 62, kLogGroupsTook = 1ull << 63;
+
 // Scratch of the fallback launch's group stage (k_chain), written and read
 // within one launch.
 struct GrpCtl {

@@ -170,3 +170,44 @@ def test_epochs_of_one_launch_do_not_wrap():
         # two products and a sum
         np.testing.assert_allclose(kre + 1j * kim, want, rtol=0, atol=2e-15)
     st.close()
+
+
+def chain_flags(nq, init, runs, cap, eps=1e-14, lay=4):
+    """The profile flags of the fallback launches that had something to do."""
+    st = sps.SparseState(nq, cap)
+    for o, v in ((sps.SPS_OPT_SMALL_RUN_CAP, 0), (sps.SPS_OPT_EXPAND, 0),
+                 (sps.SPS_OPT_LAYER_GATES, lay), (sps.SPS_OPT_PROFILE, 1)):
+        st.set_option(o, v)
+    st.set_amplitudes(*init)
+    for g in runs:
+        st.apply(W.to_array(g), eps)
+    out = [(r["flags"], r["n_in"], r["n_out"]) for r in st.profile_read() if r["kind"] == 11 and r["n_in"]]
+    try:
+        st.sync()
+    except sps.SpsError as e:
+        assert e.status == sps.SPS_ERR_CAPACITY
+    st.close()
+    return out
+
+
+@pytest.mark.parametrize("kind,gates,took", [("givens", 3, True), ("givens", 6, True), ("controlled", 4, True),
+                                             ("all", 3, True), ("all", 6, True), ("all", 7, False),
+                                             ("all", 2, False)])
+@pytest.mark.parametrize("nq,count", [(14, 700), (63, 2500), (100, 900)])
+def test_which_runs_are_taken_as_groups(kind, gates, took, nq, count):
+    rng = W.SplitMix64(nq + gates)
+    init = random_state(nq, count, count)
+    recs = chain_flags(nq, init, [layer(nq, kind, gates, rng)], 1 << 17)
+    assert len(recs) == 1 and recs[0][1] == count
+    assert bool(recs[0][0] & 64) == took and count < recs[0][2] <= 1 << 17
+
+
+def test_members_over_the_capacity_are_handed_back():
+    """640 labels with 8 members each: taken at a capacity of 5,120, not of 5,119
+    (where the passes find the error)."""
+    init = random_state(20, 640, 5)
+    run = [W.H(15), W.H(16), W.H(17)]
+    (flags, _, n), = chain_flags(20, init, [run], 5120, lay=1)
+    assert flags & 64 and n == 5120
+    (flags, _, n), = chain_flags(20, init, [run], 5119, lay=1)
+    assert not flags & 64 and flags & 128 and n == 2560
