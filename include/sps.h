@@ -356,7 +356,8 @@ typedef enum sps_option {
                                   one butterfly per group of labels that the
                                   active gates' flips connect (up to 64 members,
                                   absent ones counted, all groups within the
-                                  capacity); 0: each
+                                  capacity; after runs where that did not hold
+                                  the next 1, 2, 4 .. 64 are not tried); 0: each
                                   pass as its own launches */,
   SPS_OPT_READOUT_MIN_PLANES = 22 /* 8 (default): a registered readout
                                   (sps_set_readout) is summed by the compiled

@@ -591,7 +591,7 @@ sps_status sps_create(uint32_t nqubits, uint64_t capacity, void* cuda_stream, sp
             (s->kw == 1 || cudaMemsetAsync(b0.hi, 0, 8, s->stream) == cudaSuccess) &&
             cudaMemcpyAsync(b0.re, &kOne, 8, cudaMemcpyHostToDevice, s->stream) == cudaSuccess &&
             cudaMemsetAsync(b0.im, 0, 8, s->stream) == cudaSuccess &&
-            cudaMemsetAsync(s->ctl, 0, sizeof(Ctl), s->stream) == cudaSuccess;
+            cudaMemsetAsync(s->ctl, 0, ctl_bytes + sizeof(GrpCtl), s->stream) == cudaSuccess;
   if (!ok) return fail(SPS_ERR_CUDA);
   LaunchCfg lc = cfg_of(s);
   if (launch_itab_clear(lc, s->itab, 1ull << s->itab_log2) < 0 ||

@@ -1486,7 +1486,12 @@ __global__ void __launch_bounds__(256, SPS_AMP_MIN_BLOCKS) k_amp_layer(Ctl* ctl,
 // label activating more than 6 gates, leaders or all members of all groups not
 // fitting the capacity, a full index) nothing is published and the passes run:
 // in particular every intermediate state of the run fits the capacity if all
-// members do, so a capacity error is the passes' to find.
+// members do, so a capacity error is the passes' to find. Runs that follow one
+// handed back skip the stage: 1, then 2, 4 .. 64 of them, as attempts are skipped
+// (GrpCtl::skip); a run with more than 6 gates that every label activates is not
+// tried. (A layer of 12 Givens on 735,471 labels of 24 qubits with 8 particles:
+// 1,415 us with the stage tried each time, 1,380 now; 7 H on 100,000 labels and
+// back: 4.25 and 3.89 ms.)
 // One build, two lookups a label and one store a survivor replace a build, 2^4
 // lookups a label and a store for every four gates: a layer of 32 Givens on the
 // 635,376-label sector took 1,160 us as eight such passes.
@@ -1959,16 +1964,21 @@ __device__ __forceinline__ uint32_t step_masks(const ChainStep& st) {
 }
 
 // The steps' gates as groups (GrpArgs); true if that produced the state. Every
-// block calls it; what decides is read after grid barriers, so all agree.
+// block calls it; what decides is read after grid barriers, so all agree. tried:
+// false if the run was not to be tried (skip: GrpCtl::skip, which block 0 changes
+// after the next barrier, when every block has read it).
 template <int KW>
 __device__ __forceinline__ bool chain_groups(Ctl* ctl, Bufs bufs, unsigned long long* itab,
-                                             GrpCtl* g, const ChainArgs& a, uint64_t n) {
+                                             GrpCtl* g, const ChainArgs& a, uint64_t n,
+                                             bool& tried, uint32_t& skip) {
   __shared__ AmpGate sg[kMaxAmpGates];
   __shared__ uint32_t splanes[8][128];
   __shared__ uint32_t sqi[8][kAmpMaxActive][kAmpRing];
   __shared__ uint32_t sqa[8][kAmpMaxActive][kAmpRing];
   __shared__ AmpLeft left;
-  if (__syncthreads_or(ctl->status != 0u)) return false;
+  skip = __ldcg(&g->skip);
+  if (__syncthreads_or(ctl->status != 0u || skip != 0u)) return false;
+  tried = true;
   const GrpArgs& ga = a.grp;
   const unsigned warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
@@ -2023,6 +2033,7 @@ __device__ __forceinline__ bool chain_groups(Ctl* ctl, Bufs bufs, unsigned long 
           ctl->amp_backoff = closure > n ? 1u : 0u;
         }
         g->took = 1u;
+        g->streak = 0u;
       }
     }
   }
@@ -2060,7 +2071,9 @@ __global__ void __launch_bounds__(256) k_chain(Ctl* ctl, Bufs bufs, unsigned lon
   if (plog && blockIdx.x == 0 && threadIdx.x == 0) plog[0] = n0;
   uint32_t serial = 0;
   uint64_t tag = 0;
-  const bool grouped = GRP && chain_groups<KW>(ctl, bufs, itab, g, a, n0);
+  bool tried = false;
+  uint32_t skip = 0u;
+  const bool grouped = GRP && chain_groups<KW>(ctl, bufs, itab, g, a, n0, tried, skip);
   for (uint32_t k = 0; k < a.nsteps && !grouped; ++k) {
     const ChainStep& st = a.steps[k];
     serial = step_serial(st);
@@ -2074,6 +2087,15 @@ __global__ void __launch_bounds__(256) k_chain(Ctl* ctl, Bufs bufs, unsigned lon
       grid_barrier(ctl, serial, tag);
       gather_emit<KW>(ctl, bufs, itab, st.g, nullptr);
     }
+    if (GRP && k == 0u && blockIdx.x == 0 && threadIdx.x == 0) {   // the run was not taken
+      if (skip) {
+        g->skip = skip - 1u;
+      } else if (tried) {
+        const uint32_t sk = g->streak;
+        g->skip = 1u << (sk < 6u ? sk : 6u);
+        g->streak = sk + 1u;
+      }
+    }
     // (nothing of this launch reads the last pass's state, unless ...)
     if (k + 1u < a.nsteps || a.w.ngates || plog) grid_barrier(ctl, serial, tag);
   }
@@ -2082,7 +2104,7 @@ __global__ void __launch_bounds__(256) k_chain(Ctl* ctl, Bufs bufs, unsigned lon
     grid_barrier(ctl, serial + 1u, tag);
   }
   if (plog && blockIdx.x == 0 && threadIdx.x == 0)
-    plog[1] = ctl->nnz | (GRP ? kLogGroupsTried : 0ull) | (grouped ? kLogGroupsTook : 0ull);
+    plog[1] = ctl->nnz | (tried ? kLogGroupsTried : 0ull) | (grouped ? kLogGroupsTook : 0ull);
 }
 
 // The barrier's bounded wait, exercised: `rounds` barriers over the grid; block
@@ -2208,17 +2230,22 @@ int launch_chain(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
     ga.load_pct = lay ? steps[0].lay.load_pct : steps[0].br.load_pct;
     ga.max_log2 = lay ? steps[0].lay.max_log2 : steps[0].br.max_log2;
     ga.capacity = lay ? steps[0].lay.capacity : steps[0].br.capacity;
+    uint32_t everywhere = 0;   // gates that every label activates
     for (uint32_t k = 0; k < nsteps; ++k) {
       const bool l = steps[k].kind == PASS_LAYER;
       const uint32_t nd = l ? steps[k].lay.d : 1u;
-      for (uint32_t q = 0; q < nd; ++q) ga.words_act |= act_words(l ? steps[k].lay.ops[q] : steps[k].br.op);
+      for (uint32_t q = 0; q < nd; ++q) {
+        const BranchOp& op = l ? steps[k].lay.ops[q] : steps[k].br.op;
+        ga.words_act |= act_words(op);
+        everywhere += (op.c[0] | op.c[1]) == 0ull && !op.givens ? 1u : 0u;
+      }
       ga.d += nd;
     }
     // one gate: the gather pass indexes only the labels with a partner and
     // reads half as much (90 us against 160 at 700,000 entries, 38 against 52
     // at 115,000); two in one layer pass: about equal (94 and 116, 206 and 163);
     // three: 350 against 206; the eight passes of a layer of 32: 1,160 and 220
-    if (ga.d < 3u || ga.d > kMaxAmpGates) ga.on = 0u;
+    if (ga.d < 3u || ga.d > kMaxAmpGates || everywhere > kAmpMaxActive) ga.on = 0u;
   }
   a.w.words = reinterpret_cast<const uint4*>(w.words);
   a.w.ftab = reinterpret_cast<const double2*>(w.ftab);

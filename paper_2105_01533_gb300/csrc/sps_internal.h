@@ -402,7 +402,7 @@ struct Ctl {
 constexpr unsigned long long kLogGroupsTried = 1ull << 62, kLogGroupsTook = 1ull << 63;
 
 // Scratch of the fallback launch's group stage (k_chain), written and read
-// within one launch.
+// within one launch (skip and streak, zero at first, are kept between launches).
 struct GrpCtl {
   unsigned long long grown;     // entries appended as leaders (some given up again)
   unsigned long long closure;   // members of all groups, and entries no gate touches
@@ -411,6 +411,8 @@ struct GrpCtl {
   unsigned long long chunk;     // next chunk of 32 entries
   unsigned int bad;             // the form does not hold
   unsigned int took;            // it produced the state
+  unsigned int skip;            // runs still to skip after some that were handed back
+  unsigned int streak;          // runs handed back in a row
   unsigned long long lm[kMaskStripes][4];   // label masks of the entries written
 };
 

@@ -5,6 +5,8 @@ it hands the run back (groups over 64 members, members over the capacity)
 and where absent members, pruned values, stored zeros, appended leaders and
 partial rounds meet."""
 
+import itertools
+
 import numpy as np
 import pytest
 
@@ -211,3 +213,33 @@ def test_members_over_the_capacity_are_handed_back():
     assert flags & 64 and n == 5120
     (flags, _, n), = chain_flags(20, init, [run], 5119, lay=1)
     assert not flags & 64 and flags & 128 and n == 2560
+
+
+def sector(nq, k):
+    lo = np.array([sum(1 << q for q in c) for c in itertools.combinations(range(nq), k)], np.uint64)
+    rng = np.random.default_rng(k)
+    lo = rng.permutation(lo)
+    return [np.zeros_like(lo), lo, rng.normal(size=len(lo)), rng.normal(size=len(lo))]
+
+
+def test_runs_that_cannot_be_taken_are_seldom_tried():
+    """Givens layers where some labels activate more than 6 gates and some do not
+    (16 qubits, 8 particles): handed back, then 1, 2, 4 .. runs are not tried.
+    Seven gates that every label activates: never tried. The state is the passes'."""
+    init = sector(16, 8)
+    run = [W.Givens(q, q + 8, 0.2 + 0.1 * q) for q in range(8)]
+    recs = chain_flags(16, init, [run] * 21, 1 << 14)
+    assert len(recs) == 21 and not any(f & 64 for f, _, _ in recs)
+    assert [i for i, (f, _, _) in enumerate(recs) if f & 128] == [0, 2, 5, 10, 19]
+    both(16, init, [run] * 3, 1e-14, 1 << 14)
+    rng = W.SplitMix64(5)
+    recs = chain_flags(14, random_state(14, 700, 2), [layer(14, "all", 7, rng)] * 3, 1 << 14)
+    assert recs and not any(f & 192 for f, _, _ in recs)
+
+
+def test_a_run_that_holds_is_taken_after_one_that_does_not():
+    init = sector(16, 8)
+    bad = [W.Givens(q, q + 8, 0.2 + 0.1 * q) for q in range(8)]
+    good = [[W.Givens(q, q + 8, 0.2 + 0.1 * q) for q in range(4)] + [W.H(16 + j)] for j in range(2)]
+    recs = chain_flags(20, init, [bad] + good, 1 << 16)
+    assert [f & 192 for f, _, _ in recs] == [128, 0, 192]
