@@ -1409,6 +1409,7 @@ __global__ void __launch_bounds__(256, SPS_AMP_MIN_BLOCKS) k_amp_layer(Ctl* ctl,
         __syncwarp();
         const uint32_t per = 32u >> (c < 5u ? c : 5u);   // groups per round
         while (qtail[c - 1] - qhead[c - 1] >= per) {
+          if (__any_sync(FULL, bad)) break;   // (32 more rounds of 32 members: 160 us)
           amp_round<KW, REAL, POST>(a, sg, spar, pl, fsm, s, out, itab, mask, ep, eps_bits, c,
                                     sqi[warp][c - 1], sqa[warp][c - 1], qhead[c - 1], per, lane,
                                     bad, written, hic);
