@@ -2049,12 +2049,16 @@ __device__ __forceinline__ bool chain_groups(Ctl* ctl, Bufs bufs, unsigned long 
   return __ldcg(&g->took) != 0u;
 }
 
-// GRP: with the group stage (its own instance: the stage's registers would
-// leave the passes two blocks an SM instead of three).
-template <int KW, bool GRP>
-__global__ void __launch_bounds__(256) k_chain(Ctl* ctl, Bufs bufs, unsigned long long* itab,
-                                               GrpCtl* g, const __grid_constant__ ChainArgs a,
-                                               unsigned long long* plog) {
+// GRP: with the group stage. BLOCKS: resident blocks an SM that the registers are
+// kept to. Inlined beside each other the stages take 114 to 128 registers (a
+// step's gate comes from a changing place in the parameters, so its words sit in
+// registers), two blocks; three blocks are 80 with 70 to 230 bytes spilled. See
+// chain_kernel for which is taken.
+template <int KW, bool GRP, int BLOCKS>
+__global__ void __launch_bounds__(256, BLOCKS) k_chain(Ctl* ctl, Bufs bufs,
+                                                       unsigned long long* itab, GrpCtl* g,
+                                                       const __grid_constant__ ChainArgs a,
+                                                       unsigned long long* plog) {
   const uint64_t n0 = ctl->nnz;
   if (amp_took(ctl, 1u)) {
     // every skipped emit copies its input's masks to its output buffer and
@@ -2215,6 +2219,25 @@ static int blocks_per_sm(int threads, size_t smem) {
   });
 }
 
+// The instance of k_chain and its resident blocks an SM. Three blocks hide more of
+// the lookups of layer passes of large states: layers of 12 Givens on 735,471 and
+// 346,104 labels 1,380 and 780 us with two, 1,270 and 710 with three; 7 H on
+// 100,000 labels and back 3.9 and 3.4 ms. Passes of one gate, small states and
+// the group stage are 2 to 10 % faster with two (a run of more gates than the
+// stage's groups hold is more often the passes').
+struct ChainKernel { const void* fn; int per_sm; };
+template <int KW, bool GRP, int BLOCKS>
+static ChainKernel chain_instance(int threads) {
+  return {(const void*)k_chain<KW, GRP, BLOCKS>, blocks_per_sm<k_chain<KW, GRP, BLOCKS>>(threads, 0)};
+}
+static ChainKernel chain_kernel(int key_words, bool groups, bool many, int threads) {
+  if (key_words == 1)
+    return groups ? (many ? chain_instance<1, true, 3>(threads) : chain_instance<1, true, 2>(threads))
+                  : (many ? chain_instance<1, false, 3>(threads) : chain_instance<1, false, 2>(threads));
+  return groups ? (many ? chain_instance<2, true, 3>(threads) : chain_instance<2, true, 2>(threads))
+                : (many ? chain_instance<2, false, 3>(threads) : chain_instance<2, false, 2>(threads));
+}
+
 int launch_chain(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
                  unsigned long long* itab, GrpCtl* grp, uint32_t grp_epoch,
                  const ChainStepDesc* steps, uint32_t nsteps, const ChainWalk& w,
@@ -2264,16 +2287,15 @@ int launch_chain(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
   for (uint32_t c = 0; c < 2 * w.npar; ++c) a.w.par[c] = w.par[c];
   const int threads = lc.threads < 256 ? lc.threads : 256;
   const int sms = lc.max_blocks * lc.threads / 2048;
-  const bool gr = a.grp.on != 0u;
-  const int per_sm = key_words == 1
-                         ? (gr ? blocks_per_sm<k_chain<1, true>>(threads, 0) : blocks_per_sm<k_chain<1, false>>(threads, 0))
-                         : (gr ? blocks_per_sm<k_chain<2, true>>(threads, 0) : blocks_per_sm<k_chain<2, false>>(threads, 0));
-  if (per_sm <= 0 || sms <= 0) return 0;
-  const int blocks = grid_of(nnz_bound, threads, per_sm * sms < 0x7FFF ? per_sm * sms : 0x7FFF);
+  uint32_t layered = 0;   // gates of layer passes
+  for (uint32_t k = 0; k < nsteps; ++k) layered += steps[k].kind == PASS_LAYER ? steps[k].lay.d : 0u;
+  const ChainKernel kern = chain_kernel(key_words, a.grp.on != 0u,
+                                        layered > kAmpMaxActive && nnz_bound >= (1ull << 20), threads);
+  if (kern.per_sm <= 0 || sms <= 0) return 0;
+  const int blocks =
+      grid_of(nnz_bound, threads, kern.per_sm * sms < 0x7FFF ? kern.per_sm * sms : 0x7FFF);
   void* args[] = {&ctl, &bufs, &itab, &grp, &a, &plog};
-  const void* kern = key_words == 1 ? (gr ? (const void*)k_chain<1, true> : (const void*)k_chain<1, false>)
-                                    : (gr ? (const void*)k_chain<2, true> : (const void*)k_chain<2, false>);
-  const cudaError_t e = cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3(threads), args, 0,
+  const cudaError_t e = cudaLaunchCooperativeKernel(kern.fn, dim3(blocks), dim3(threads), args, 0,
                                                     (cudaStream_t)lc.stream);
   if (e != cudaSuccess) {
     cudaGetLastError();

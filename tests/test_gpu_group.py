@@ -243,3 +243,21 @@ def test_a_run_that_holds_is_taken_after_one_that_does_not():
     good = [[W.Givens(q, q + 8, 0.2 + 0.1 * q) for q in range(4)] + [W.H(16 + j)] for j in range(2)]
     recs = chain_flags(20, init, [bad] + good, 1 << 16)
     assert [f & 192 for f, _, _ in recs] == [128, 0, 192]
+
+
+@pytest.mark.parametrize("kind", ["givens", "all"])
+@pytest.mark.parametrize("nq", [20, 100])
+def test_large_bounds_take_the_instances_of_three_blocks(kind, nq):
+    """Seven gates on 9,000 labels with a bound past 2^20, with the group stage
+    (tried, then skipped) and without."""
+    rng = W.SplitMix64(nq)
+    init = random_state(nq, 9000, 4)
+    parts = [layer(nq, kind, 7, rng) + [W.T(1)] for _ in range(2)]
+    err, got = both(nq, init, parts, 1e-14, 1 << 21)
+    assert err is None
+    orc = OracleState(nq)
+    orc.set(*init)
+    for g in parts:
+        orc.apply(W.to_array(g), eps=1e-14)
+    # amplitudes of modulus up to 4, seven butterflies twice: some 60 roundings
+    compare_states(got, orc.get(), 1e-14, atol=1e-12)
