@@ -76,3 +76,50 @@ def test_gather_equals_scatter(nq, count, load):
     for a, b in zip(got[:half], got[half:]):
         for x, y in zip(a, b):
             np.testing.assert_array_equal(x, y)
+
+
+def index_load(active, n, load):
+    """Labels over slots of the gather index for n entries: at most 2 n * load slots
+    counted in entries, doubled below 2^22 slots."""
+    lg = 8
+    while (1 << lg) * load < 100 * n:
+        lg += 1
+    return active / (1 << (lg + 1 if lg < 22 else lg))
+
+
+def large_state(nq, count):
+    """As state, with up to 2^24 distinct labels."""
+    rng = np.random.default_rng(count)
+    i = np.arange(count, dtype=np.uint64)
+    lo = (((i >> np.uint64(1)) * np.uint64(2654435761)) % np.uint64(1 << 23)) << np.uint64(1) | (i & np.uint64(1))
+    lo[::5] ^= np.uint64(1 << 26)
+    hi = np.zeros_like(lo)
+    if nq > 64:
+        hi = lo & np.uint64(63)
+        lo = lo >> np.uint64(3) | (lo & np.uint64(7)) << np.uint64(61)
+    return hi, lo, rng.normal(size=count), rng.normal(size=count)
+
+
+@pytest.mark.parametrize("nq,count", [(30, 3_700_000), (70, 3_650_001)])
+def test_gather_equals_scatter_in_a_crowded_index(nq, count):
+    """87 and 88 % of 2^22 slots taken: claims are carried through several buckets,
+    past the end of the table too."""
+    assert 0.86 < index_load(count, count, 90) < 0.89
+    init = large_state(nq, count)
+    t = 7 if nq < 64 else 66
+    gates = [W.H(0), W.Givens(0, t, 1.1), W.Ry(t, 0.3)]
+    got = []
+    for form in (1, 2):
+        st = sps.SparseState(nq, 2 * count + 64)
+        for o, v in ((sps.SPS_OPT_SMALL_RUN_CAP, 0), (sps.SPS_OPT_EXPAND, 0), (sps.SPS_OPT_AMP_ONLY, 0),
+                     (sps.SPS_OPT_LAYER_GATES, 1), (sps.SPS_OPT_BRANCH_FORM, form),
+                     (sps.SPS_OPT_LOAD_FACTOR_PCT, 90 if form == 2 else 50)):
+            st.set_option(o, v)
+        for g in gates:   # every label is indexed for H and Ry
+            st.set_amplitudes(*init)
+            st.apply(W.to_array([g]), 0.0)
+            got.append(st.get_amplitudes() + (st.updates(),))
+        st.close()
+    for a, b in zip(got[:3], got[3:]):
+        for x, y in zip(a, b):
+            np.testing.assert_array_equal(x, y)
