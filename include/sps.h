@@ -202,10 +202,11 @@ sps_status sps_set_readout(sps_state* s, const uint64_t mask[2], const uint64_t 
  * P|j> = i^nY (-1)^popcount(j & z) |j ^ x> (nY = number of Y factors), a label
  * j with every control set goes to cos(theta/2)|j> - i sin(theta/2) P|j>.
  * A string with X or Y factors is one branching pass on the pairs (j, j ^ x)
- * (Sec. 3.1), pruned with prune_eps; a string of Z factors only is diagonal
- * and runs as a fused run (a CNOT ladder onto one z qubit, Rz, the ladder
- * undone). Enqueues only, like sps_apply; counts as one gate for the update
- * counter (the diagonal form counts its ladder). Errors: SPS_ERR_ARG for an
+ * (Sec. 3.1), pruned with prune_eps; a string of Z factors only is diagonal:
+ * one kernel that multiplies each label's amplitude by the phase of its parity
+ * and counts as the fused run it stands for (a CNOT ladder onto one z qubit,
+ * Rz, the ladder undone). Enqueues only, like sps_apply; counts as one gate for
+ * the update counter (the diagonal form counts its ladder). Errors: SPS_ERR_ARG for an
  * empty string, masks beyond nqubits, controls on the string or a non-finite
  * theta; device errors as for sps_apply (the failing gate is reported as 0). */
 sps_status sps_pauli_exp(sps_state* s, const uint64_t x[2], const uint64_t z[2],
@@ -308,7 +309,7 @@ typedef enum sps_option {
   SPS_OPT_FUSED_LABELS = 17    /* labels each thread of a direct fused pass walks
                                   together (sharing each op's decode): 1, 2, 4
                                   or 8; 0 (default) picks the most that still
-                                  leave about four warps per SM */,
+                                  leave 32 warps per SM */,
   SPS_OPT_AMP_ONLY = 18        /* 1 (default): a gather-form branching pass (one
                                   gate, or a layer pass) first tries the
                                   amplitude-only form: if every active label

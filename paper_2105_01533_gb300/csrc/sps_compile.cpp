@@ -856,8 +856,13 @@ bool build_bitslice_expand(const Pass& ex, const Pass& run, uint32_t nqubits, do
   }
   comb.phases.insert(comb.phases.end(), run.phases.begin(), run.phases.end());
   if (comb.phases.size() > kMaxFusedPhases + kMaxExpandGates) return false;
-  // products of chunk entries keep 2^-61 of the common factor's modulus: enough
-  // where every slot's factor has modulus one, not for rotations in the head
+  // A product of chunk entries drops two bits of scale: with n chunks a unit is
+  // 2^-(62 - 2 (n - 1)) of the common factor's power of two, and an output is off
+  // by a few. Against exact products that is 2^-53.3 of the output's modulus with
+  // two chunks and 2^-52.9 with four; as an expansion and a run, whose last
+  // product is in FP64, 2^-52.6 and 2^-52.4. That holds where every slot's factor
+  // has modulus one: rotations in the head may make an output any amount smaller
+  // than the common factor.
   if (base > 0 && aux_bits_of(comb.ops) > kBsDirectBits) return false;
   if (!build_bitslice_rows(comb, nqubits, targets, true, out)) return false;
   out->expand = true;
