@@ -388,3 +388,36 @@ def test_readers_and_writers_after_runs_that_keep_labels(n):
     assert upd == upd0
     compare_states(last, last0, 1e-14)
     np.testing.assert_allclose(seen, seen0, rtol=0, atol=1e-12)
+
+
+@pytest.mark.parametrize("nq,blocks", [(20, 1), (20, 5), (40, 152), (40, 153), (40, 608), (63, 609), (64, 31),
+                                       (100, 1217)])
+def test_few_entries_under_a_large_bound(nq, blocks):
+    """Small chunks: runs applied one after the other without a wait, so the bound
+    (and the grid) grows past the count, on labels that keep every member: against
+    the out-of-place passes, bit for bit, attempts taken."""
+    rng = np.random.default_rng(blocks)
+    top = rng.permutation(1 << 12)[:blocks].astype(np.uint64)
+    lab = (np.repeat(top, 16) << np.uint64(4)) | np.tile(np.arange(16, dtype=np.uint64), blocks)
+    hi, lo = np.zeros_like(lab), lab
+    if nq > 64:
+        hi, lo = lab >> np.uint64(8), (lab & np.uint64(255)) << np.uint64(56)
+    init = (hi, lo, rng.normal(size=len(lab)), rng.normal(size=len(lab)))
+    q0 = 56 if nq > 64 else 0
+    run = W.to_array([W.Ry(q0, 0.3), W.Rx(q0 + 1, 1.1), W.H(q0 + 2)] +
+                     [W.Ry(q0 + 3, 0.7, q0 + 6), W.T(q0 + 1)])
+    got = []
+    for amp in (1, 0):
+        st = sps.SparseState(nq, 1 << 20)
+        for o, v in ((sps.SPS_OPT_SMALL_RUN_CAP, 0), (sps.SPS_OPT_EXPAND, 0), (sps.SPS_OPT_AMP_ONLY, amp),
+                     (sps.SPS_OPT_BITSLICE_MIN_OPS, 0), (sps.SPS_OPT_PROFILE, 1)):
+            st.set_option(o, v)
+        st.set_amplitudes(*init)
+        for _ in range(6):
+            st.apply(run, 1e-14)
+        if amp:
+            assert all(r["n_out"] for r in st.profile_read() if r["kind"] == 10)
+        got.append(st.get_amplitudes() + (st.updates(),))
+        st.close()
+    for x, y in zip(*got):
+        np.testing.assert_array_equal(x, y)
