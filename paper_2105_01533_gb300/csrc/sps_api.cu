@@ -1144,6 +1144,16 @@ static sps_status build_plan(sps_state* s, const sps_gate* gates, size_t ngates,
     P->bs_tab_entries += P->bs_ex.table_entries();
   }
   std::vector<unsigned char>& img = P->image;
+  {   // its size at most (grown piece by piece it was copied over and over)
+    size_t most = bs_bytes;
+    for (size_t i = 0; i < np; ++i) {
+      const Pass& p = passes[i];
+      most += p.words.size() * sizeof(OpWord) + p.ftab.size() * sizeof(double) +
+              p.ex_f.size() * sizeof(double) + p.ex_m.size() * sizeof(uint64_t) +
+              sizeof(BranchOp) + sizeof(RunPass) + 5 * 16;
+    }
+    img.reserve(most);
+  }
   img.assign(bs_bytes, 0);
   for (size_t i = 0; i < np; ++i) {
     const BsPass& b = P->bs[i];

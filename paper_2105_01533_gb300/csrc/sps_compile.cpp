@@ -576,6 +576,7 @@ void encode_ops(Pass* p) {
   };
   std::vector<Prim> prims;
   prims.reserve(2 * ops.size());
+  bool high = false;   // some op reads or flips qubits 64..127
   uint32_t reads[128] = {}, writes[128] = {};   // per qubit: first level after its last
                                                 // reader, its last flip
   uint32_t levels = 0;
@@ -599,6 +600,7 @@ void encode_ops(Pass* p) {
       }
     }
     levels = std::max(levels, after);
+    high = high || (c[1] | (flip ? t1 : 0ull)) != 0;
     prims.push_back(q);
   };
   // fire slots in op order; slot k's factor is the phase its op applies
@@ -653,9 +655,11 @@ void encode_ops(Pass* p) {
     // A level's flips within the low 64 qubits come first, as a level of their own:
     // they take half the words where enough of them come together. (Its phase ops
     // follow all its flips, which may flip what they read.)
-    levels *= 2;
-    for (Prim& q : prims)
-      q.level = 2 * q.level + (!q.flip || (q.c[1] | q.t[1]) != 0 ? 1u : 0u);
+    if (high) {
+      levels *= 2;
+      for (Prim& q : prims)
+        q.level = 2 * q.level + (!q.flip || (q.c[1] | q.t[1]) != 0 ? 1u : 0u);
+    }
     std::vector<uint32_t> count(2 * (size_t)levels, 0u);
     std::vector<uint8_t> wide(levels, 0);
     for (const Prim& q : prims) {
@@ -663,7 +667,7 @@ void encode_ops(Pass* p) {
       if (q.c[1] | (q.flip ? q.t[1] : 0ull)) wide[q.level] = 1;
     }
     auto pairs = [&](uint32_t h) { return (count[h] + 1u) / 2u; };
-    for (uint32_t l = 0; l < levels;) {   // narrow stretches shorter than this many steps
+    for (uint32_t l = 0; high && l < levels;) {   // narrow stretches shorter than this many steps
       constexpr uint32_t kMinNarrow = 8;
       uint32_t e = l, steps = 0;
       for (; e < levels && !wide[e]; ++e) steps += pairs(2 * e) + pairs(2 * e + 1);
@@ -671,7 +675,7 @@ void encode_ops(Pass* p) {
       l = e + 1;
     }
     for (Prim& q : prims)   // both halves wide: one level
-      if (!(q.level & 1u) && wide[q.level] && wide[q.level + 1]) {
+      if (high && !(q.level & 1u) && wide[q.level] && wide[q.level + 1]) {
         --count[2 * q.level];
         ++count[2 * ++q.level];
       }
