@@ -253,10 +253,9 @@ void sps::hook_free(void* p, size_t bytes, void* stream) {
   f(ctx, p, (bytes + 255) & ~size_t(255), stream);
 }
 
-double* sps::device_view(const void* p, int device, bool host_too) {
+static double* view_on(const void* p, int device, int current, bool host_too) {
   cudaPointerAttributes at;
-  int current = -1;
-  if (cudaGetDevice(&current) != cudaSuccess || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();
     return nullptr;
   }
@@ -267,6 +266,24 @@ double* sps::device_view(const void* p, int device, bool host_too) {
                           reinterpret_cast<uintptr_t>(at.devicePointer), host_too)
              ? static_cast<double*>(at.devicePointer)
              : nullptr;
+}
+
+static int current_device() {
+  int current = -1;
+  if (cudaGetDevice(&current) != cudaSuccess) cudaGetLastError();
+  return current;
+}
+
+double* sps::device_view(const void* p, int device) {
+  return view_on(p, device, current_device(), true);
+}
+
+bool sps::device_arrays(int device, const void* hi, const void* lo, const void* re,
+                        const void* im) {
+  const int current = current_device();
+  for (const void* p : {lo, re, im, hi})
+    if (p && !view_on(p, device, current, false)) return false;
+  return true;
 }
 
 namespace {
@@ -1550,9 +1567,7 @@ sps_status sps_get_amplitudes(sps_state* s, uint64_t* key_hi, uint64_t* key_lo, 
   if (!s || !key_lo || !re || !im || !nnz_out) return SPS_ERR_ARG;
   // into device arrays one kernel copies the state before the one wait, which
   // tells whether it did (see copy_entries)
-  const bool exported = device_view(key_lo, s->device, false) &&
-                        device_view(re, s->device, false) && device_view(im, s->device, false) &&
-                        (!key_hi || device_view(key_hi, s->device, false));
+  const bool exported = device_arrays(s->device, key_hi, key_lo, re, im);
   sps_status st = SPS_OK;
   if (exported) {
     st = flush_reset(s);
@@ -1733,7 +1748,7 @@ sps_status sps_probability_async(sps_state* s, const uint64_t mask[2], const uin
   if (fs != SPS_OK) return fs;
   const LaunchCfg lc = cfg_of(s);
   // the kernel writes the caller's word itself where it can
-  double* direct = device_view(out, s->device, true);
+  double* direct = device_view(out, s->device);
   ProfScope ps(s, 12, s->pass_serial, 0, 0u);
   const int pn = launch_probability(lc, s->kw, s->ctl, s->bufs, mask[0], mask[1], value[0],
                                     value[1], s->partials, prob_grid(s),
@@ -1818,7 +1833,7 @@ sps_status sps_measure(sps_state* s, uint32_t qubit, double r, double* out) {
   const uint32_t serial = ++s->pass_serial;
   s->amp_force = true;   // the collapse moves labels
   ProfScope ps(s, 8, serial, 1, 1u);
-  double* direct = device_view(out, s->device, true);
+  double* direct = device_view(out, s->device);
   const int n = launch_measure(lc, s->kw, s->ctl, s->bufs, qubit, r, s->partials, s->prob_blocks,
                                s->dmeasure, direct, s->nnz_bound, s->masks.writer(), ps.slot);
   ps.done();

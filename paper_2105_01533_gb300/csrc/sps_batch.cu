@@ -551,8 +551,7 @@ sps_status sps_batch_get_amplitudes(sps_batch* b, uint32_t index, uint64_t* key_
   if (d.nnz > cap) return SPS_ERR_CAPACITY;
   if (d.nnz == 0) return SPS_OK;
   const unsigned c = d.cur;
-  if (device_view(key_lo, b->device, false) && device_view(re, b->device, false) &&
-      device_view(im, b->device, false) && (!key_hi || device_view(key_hi, b->device, false))) {
+  if (device_arrays(b->device, key_hi, key_lo, re, im)) {
     const SoA s{d.lo[c], d.kw == 2 ? d.hi[c] : nullptr, d.re[c], d.im[c]};
     if (launch_copy_entries(b->stream, s, d.nnz, key_hi, key_lo, re, im) < 0)
       return cuda_st(cudaGetLastError());

@@ -660,7 +660,9 @@ inline bool kernel_may_write(MemKind kind, int owner, int device, int current, u
   return kind == MEM_DEVICE ? owner == device : kind == MEM_PINNED && host_too;
 }
 // The address at which a kernel may write the caller's words at p, or null.
-double* device_view(const void* p, int device, bool host_too);
+double* device_view(const void* p, int device);
+// Whether a kernel may write all of the caller's arrays (hi nullable), in device memory.
+bool device_arrays(int device, const void* hi, const void* lo, const void* re, const void* im);
 int launch_probability(const LaunchCfg& lc, int key_words, Ctl* ctl, Bufs bufs,
                        uint64_t mask_lo, uint64_t mask_hi, uint64_t val_lo, uint64_t val_hi,
                        double* partials, int nblocks, double* result,
