@@ -1357,8 +1357,9 @@ __global__ void __launch_bounds__(256, SPS_AMP_MIN_BLOCKS) k_amp_layer(Ctl* ctl,
 #pragma unroll
     for (uint32_t c = 0; c < kAmpMaxActive; ++c) qhead[c] = qtail[c] = 0u;
     // chunks of fewer entries where there is not one of 32 for every warp (5,000 labels
-    // that find their members absent: 32 rounds a warp, 160 us; 4 now). A vote between
-    // the rounds would do too, but large states then take 1.5 % longer.
+    // that find their members absent: 32 rounds a warp took 160 us, four take 22; 8,008
+    // that find them 26.5 and 22.5). A vote between the rounds would do too, but
+    // large states then take 1.5 % longer.
     const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
     uint32_t chunk = 32u;
     while (chunk > 1u && n <= (chunk >> 1) * warps) chunk >>= 1;
@@ -1497,7 +1498,7 @@ __global__ void __launch_bounds__(256, SPS_AMP_MIN_BLOCKS) k_amp_layer(Ctl* ctl,
 // handed back skip the stage: 1, then 2, 4 .. 64 of them, as attempts are skipped
 // (GrpCtl::skip); a run with more than 6 gates that every label activates is not
 // tried. (A layer of 12 Givens on 735,471 labels of 24 qubits with 8 particles:
-// 1,415 us with the stage tried each time, 1,380 now; 7 H on 100,000 labels and
+// 1,415 us with the stage tried each time, 1,380 so; 7 H on 100,000 labels and
 // back: 4.25 and 3.89 ms.)
 // One build, two lookups a label and one store a survivor replace a build, 2^4
 // lookups a label and a store for every four gates: a layer of 32 Givens on the
@@ -2227,8 +2228,8 @@ static int blocks_per_sm(int threads, size_t smem) {
 
 // The instance of k_chain and its resident blocks an SM. Three blocks hide more of
 // the lookups of layer passes of large states: layers of 12 Givens on 735,471 and
-// 346,104 labels 1,380 and 780 us with two, 1,270 and 710 with three; 7 H on
-// 100,000 labels and back 3.9 and 3.4 ms. Passes of one gate, small states and
+// 346,104 labels 1,400 and 785 us with two, 1,300 and 713 with three; 7 H on
+// 100,000 labels and back 3.87 and 3.37 ms. Passes of one gate, small states and
 // the group stage are 2 to 10 % faster with two (a run of more gates than the
 // stage's groups hold is more often the passes').
 struct ChainKernel { const void* fn; int per_sm; };
